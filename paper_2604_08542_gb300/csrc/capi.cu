@@ -41,6 +41,7 @@ cudaError_t gcm_qkv_backward(const void* dq, const void* dk, const void* dv, con
                              int D, float* dx, float* dwqkv, float* dbqkv, float* dw_eta, float* db_eta, void* ws,
                              int* status, int sms, cudaStream_t st);
 bool fp32_shape_supported(int D, int F);
+bool fp32_tiled_shape(int D, int F);
 bool bf16_shape_supported(int D, int F);
 bool update_shape_supported(int D, int F);
 cudaError_t launch_bprep(const Params& prm, int chains, cudaStream_t st);
@@ -204,6 +205,21 @@ bool same_layout(const Plan& p, const int64_t* off, int32_t C, const int32_t* pt
   return std::memcmp(p.seq_chunk_ptr.data(), ptr, sizeof(int32_t) * (S + 1)) == 0;
 }
 
+// The tail fill's piece-time model for the register-tiled float32 kernels, in
+// units of an applied token (forward, 0.2 us on one SM) or an apply-VJP token
+// (backward, 0.5 us); the fixed cost is the weights' load and the sums' store.
+void fp32_fill_model(Schedule& sch) {
+  sch.fill = 3;
+  sch.fill_ovh[0] = 40.f;
+  sch.fill_ovh[1] = 25.f;
+  sch.fill_ovh[2] = 20.f;
+  sch.fill_ovh[3] = 16.f;
+  sch.fill_key_tok = 1.8f;
+  sch.fill_bkey_tok = 2.07f;
+  sch.fill_bkey_sub = 0.f;
+  sch.fill_start = 10.f;
+}
+
 int ensure_plan(scal3r_ttt_handle* hd, const int64_t* off, int32_t C, const int32_t* ptr, int32_t S) {
   if (!off || !ptr || C < 0 || S < 1) return SCAL3R_ERR_INVALID_ARG;
   if (same_layout(hd->plan, off, C, ptr, S)) return SCAL3R_OK;
@@ -214,7 +230,8 @@ int ensure_plan(scal3r_ttt_handle* hd, const int64_t* off, int32_t C, const int3
     sch.align = 16;
     sch.min_tokens = 16;
   }
-  if (hd->cfg.dtype != SCAL3R_BF16 || hd->wide || hd->shape.lin) sch.fill = 0;   // its model is the BF16 kernels'
+  if (hd->cfg.dtype == SCAL3R_FP32 && fp32_tiled_shape(hd->shape.D, hd->shape.F)) fp32_fill_model(sch);
+  else if (hd->cfg.dtype != SCAL3R_BF16 || hd->wide || hd->shape.lin) sch.fill = 0;   // its model is the BF16 kernels'
   int rc = build_plan(np, hd->shape, sch, hd->num_sms, off, C, ptr, S, hd->wide ? 1 : hd->cfg.ckpt_every,
                       mse_compose);
   if (rc != SCAL3R_OK) return rc;

@@ -1,4 +1,6 @@
-// Plain FP32 SIMT path of the test-time-training layer (no tensor cores).
+// Plain FP32 SIMT path of the test-time-training layer (no tensor cores), and
+// the dispatch of the float32 path: head_dim 64 with hidden 128 runs on the
+// register-tiled kernels of fp32_tiled.cu, the small shape (16, 32) here.
 //
 // One CTA processes one work item: a token range of one chain (sequence,
 // head) at one chunk step, in tiles of TT tokens.  Fast weights sit in shared
@@ -21,19 +23,17 @@
 //          L1 += dz1 k^T, L3 += dz3 k^T, L2t += dp e^T (+ u dy^T for MSE).
 //   BAPPLY VJP of o = f_W(q): dq and L1 += dzq1 q^T, L3 += dzq3 q^T,
 //          L2t += uq do^T.
-#include <cuda_bf16.h>
-
 #include "ttt_internal.h"
 
 namespace scal3r {
+bool fp32_tiled_shape(int D, int F);
+cudaError_t prepare_fp32_tiled();
+cudaError_t launch_fp32_tiled_sweep(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st);
+cudaError_t launch_fp32_tiled_bsweep(const Params& prm, const WorkItem* items, int n, cudaStream_t st);
+
 namespace {
 
 constexpr int NTH = 256;
-
-__device__ __forceinline__ float ldio(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ float ldio(const __nv_bfloat16* p, size_t i) { return __bfloat162float(p[i]); }
-__device__ __forceinline__ void stio(float* p, size_t i, float v) { p[i] = v; }
-__device__ __forceinline__ void stio(__nv_bfloat16* p, size_t i, float v) { p[i] = __float2bfloat16_rn(v); }
 
 template <int D, int F>
 struct Geo {
@@ -61,11 +61,11 @@ __device__ void load_weights(float* ws, const float* __restrict__ w) {
   }
 }
 
-template <int D, int F, int TT, typename TIO>
-__device__ void load_rows(float* dst, const TIO* __restrict__ src, int64_t t, int n, int H, int h) {
+template <int D, int F, int TT>
+__device__ void load_rows(float* dst, const float* __restrict__ src, int64_t t, int n, int H, int h) {
   for (int i = threadIdx.x; i < TT * D; i += NTH) {
     const int r = i / D, c = i % D;
-    dst[i] = (r < n) ? ldio(src, ((size_t)(t + r) * H + h) * D + c) : 0.f;
+    dst[i] = (r < n) ? src[((size_t)(t + r) * H + h) * D + c] : 0.f;
   }
 }
 
@@ -125,7 +125,7 @@ fp32_sweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
     for (int64_t t = it.t0; t < it.t1; t += TT) {
       const int n = (int)((it.t1 - t) < TT ? (it.t1 - t) : TT);
       __syncthreads();
-      load_rows<D, F, TT, float>(Ks, q, t, n, H, h);
+      load_rows<D, F, TT>(Ks, q, t, n, H, h);
       __syncthreads();
       {
         const int f = tid % F;
@@ -168,8 +168,8 @@ fp32_sweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
   for (int64_t t = it.t0; t < it.t1; t += TT) {
     const int n = (int)((it.t1 - t) < TT ? (it.t1 - t) : TT);
     __syncthreads();
-    load_rows<D, F, TT, float>(Ks, kk, t, n, H, h);
-    load_rows<D, F, TT, float>(Vs, vv, t, n, H, h);
+    load_rows<D, F, TT>(Ks, kk, t, n, H, h);
+    load_rows<D, F, TT>(Vs, vv, t, n, H, h);
     for (int i = tid; i < TT * nr; i += NTH)
       etas[i] = (i / nr < n) ? p.lr[((size_t)(t + i / nr) * H + h) * nr + i % nr] : 0.f;
     __syncthreads();
@@ -253,7 +253,7 @@ fp32_sweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
 // backward
 // ---------------------------------------------------------------------------
 
-template <int D, int F, typename TIO>
+template <int D, int F>
 __global__ void __launch_bounds__(NTH, 1)
 fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
   using G = Geo<D, F>;
@@ -306,14 +306,14 @@ fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
 
   if (it.role == ROLE_BAPPLY) {
     load_weights<D, F>(sm, w);
-    const TIO* q = (const TIO*)p.q;
-    const TIO* go = (const TIO*)p.d_o;
-    TIO* dq = (TIO*)p.dq;
+    const float* q = (const float*)p.q;
+    const float* go = (const float*)p.d_o;
+    float* dq = (float*)p.dq;
     for (int64_t t = it.t0; t < it.t1; t += TT) {
       const int n = (int)((it.t1 - t) < TT ? (it.t1 - t) : TT);
       __syncthreads();
-      load_rows<D, F, TT, TIO>(Ks, q, t, n, H, h);
-      load_rows<D, F, TT, TIO>(Vs, go, t, n, H, h);
+      load_rows<D, F, TT>(Ks, q, t, n, H, h);
+      load_rows<D, F, TT>(Vs, go, t, n, H, h);
       __syncthreads();
       {
         const int f = tid % F;
@@ -341,7 +341,7 @@ fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
 #pragma unroll 16
           for (int f = 0; f < F; ++f)
             g = fmaf(DZ1s[i * F + f], M1[f * G::LDW + d], fmaf(DZ3s[i * F + f], M3[f * G::LDW + d], g));
-          if (i < n) stio(dq, ((size_t)(t + i) * H + h) * D + d, g);
+          if (i < n) dq[((size_t)(t + i) * H + h) * D + d] = g;
         }
       }
       {
@@ -372,18 +372,18 @@ fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
   }
 
   // ROLE_BKEY
-  const TIO* kk = (const TIO*)p.k;
-  const TIO* vv = (const TIO*)p.v;
-  TIO* dk = (TIO*)p.dk;
-  TIO* dv = (TIO*)p.dv;
+  const float* kk = (const float*)p.k;
+  const float* vv = (const float*)p.v;
+  float* dk = (float*)p.dk;
+  float* dv = (float*)p.dv;
   const bool pm = p.lr_mat != 0;
   const int nr = pm ? 3 : 1;
   for (int64_t t = it.t0; t < it.t1; t += TT) {
     const int n = (int)((it.t1 - t) < TT ? (it.t1 - t) : TT);
     __syncthreads();
     load_weights<D, F>(sm, w);
-    load_rows<D, F, TT, TIO>(Ks, kk, t, n, H, h);
-    load_rows<D, F, TT, TIO>(Vs, vv, t, n, H, h);
+    load_rows<D, F, TT>(Ks, kk, t, n, H, h);
+    load_rows<D, F, TT>(Vs, vv, t, n, H, h);
     for (int i = tid; i < TT * nr; i += NTH)
       etas[i] = (i / nr < n) ? p.lr[((size_t)(t + i / nr) * H + h) * nr + i % nr] : 0.f;
     __syncthreads();
@@ -516,7 +516,7 @@ fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
           dh = -Vs[i * D + d] * de;
         }
         DHs[i * D + d] = dh;
-        if (i < n) stio(dv, ((size_t)(t + i) * H + h) * D + d, dvv);
+        if (i < n) dv[((size_t)(t + i) * H + h) * D + d] = dvv;
       }
     }
     __syncthreads();
@@ -542,7 +542,7 @@ fp32_bsweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
 #pragma unroll 16
         for (int f = 0; f < F; ++f)
           g = fmaf(DZ1s[i * F + f], M1[f * G::LDW + d], fmaf(DZ3s[i * F + f], M3[f * G::LDW + d], g));
-        if (i < n) stio(dk, ((size_t)(t + i) * H + h) * D + d, g);
+        if (i < n) dk[((size_t)(t + i) * H + h) * D + d] = g;
       }
       for (int i = tid; i < n; i += NTH) {
         float a = 0.f;
@@ -599,61 +599,35 @@ constexpr size_t bwd_smem() {
   return sizeof(float) * (Geo<D, F>::WS + 7 * 8 * D + 15 * 8 * F + 3 * 8);
 }
 
-template <int D, int F>
-cudaError_t launch_fwd(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st) {
-  const size_t smem = fwd_smem<D, F>();
-  fp32_sweep_kernel<D, F><<<n, NTH, smem, st>>>(prm, items, step);
-  return cudaGetLastError();
-}
-
-template <int D, int F, typename TIO>
-cudaError_t launch_bwd(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st) {
-  const size_t smem = bwd_smem<D, F>();
-  fp32_bsweep_kernel<D, F, TIO><<<n, NTH, smem, st>>>(prm, items, step);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
+constexpr int SD = 16, SF = 32;   // the shape of the plain kernels
+
 cudaError_t prepare_fp32() {
-  const struct {
-    const void* f;
-    size_t smem;
-  } ks[] = {{(const void*)fp32_sweep_kernel<64, 128>, fwd_smem<64, 128>()},
-            {(const void*)fp32_sweep_kernel<16, 32>, fwd_smem<16, 32>()},
-            {(const void*)fp32_bsweep_kernel<64, 128, float>, bwd_smem<64, 128>()},
-            {(const void*)fp32_bsweep_kernel<16, 32, float>, bwd_smem<16, 32>()},
-            {(const void*)fp32_bsweep_kernel<64, 128, __nv_bfloat16>, bwd_smem<64, 128>()}};
-  for (const auto& k : ks) {
-    cudaError_t e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(fp32_sweep_kernel<SD, SF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)fwd_smem<SD, SF>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fp32_bsweep_kernel<SD, SF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)bwd_smem<SD, SF>());
+  return e == cudaSuccess ? prepare_fp32_tiled() : e;
 }
 
-bool fp32_shape_supported(int D, int F) {
-  return (D == 64 && F == 128) || (D == 16 && F == 32);
-}
+bool fp32_shape_supported(int D, int F) { return fp32_tiled_shape(D, F) || (D == SD && F == SF); }
 
 cudaError_t launch_fp32_sweep(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  if (prm.D == 64 && prm.F == 128) return launch_fwd<64, 128>(prm, items, n, step, st);
-  if (prm.D == 16 && prm.F == 32) return launch_fwd<16, 32>(prm, items, n, step, st);
-  return cudaErrorInvalidValue;
+  if (fp32_tiled_shape(prm.D, prm.F)) return launch_fp32_tiled_sweep(prm, items, n, step, st);
+  if (prm.D != SD || prm.F != SF) return cudaErrorInvalidValue;
+  fp32_sweep_kernel<SD, SF><<<n, NTH, fwd_smem<SD, SF>(), st>>>(prm, items, step);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_fp32_bsweep(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  if (prm.D == 64 && prm.F == 128) return launch_bwd<64, 128, float>(prm, items, n, step, st);
-  if (prm.D == 16 && prm.F == 32) return launch_bwd<16, 32, float>(prm, items, n, step, st);
-  return cudaErrorInvalidValue;
-}
-
-// Backward of the BF16 path on CUDA cores: bf16 token tensors, fp32 arithmetic.
-cudaError_t launch_simt_bsweep_bf16io(const Params& prm, const WorkItem* items, int n, int step, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  if (prm.D == 64 && prm.F == 128) return launch_bwd<64, 128, __nv_bfloat16>(prm, items, n, step, st);
-  return cudaErrorInvalidValue;
+  if (fp32_tiled_shape(prm.D, prm.F)) return launch_fp32_tiled_bsweep(prm, items, n, st);
+  if (prm.D != SD || prm.F != SF) return cudaErrorInvalidValue;
+  fp32_bsweep_kernel<SD, SF><<<n, NTH, bwd_smem<SD, SF>(), st>>>(prm, items, step);
+  return cudaGetLastError();
 }
 
 }  // namespace scal3r
