@@ -174,6 +174,15 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void*
                : "memory");
 }
 
+// The tile added to global memory (the map's element type).
+__device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, const void* ssrc, int32_t c0, int32_t c1,
+                                                  int32_t c2) {
+  asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(smem_u32(ssrc)), "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
+}
+
 // TMA tile load / store with a 5-D map (bulk tensor copies of strided
 // block layouts).
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, uint64_t* bar, int32_t c0,
@@ -195,6 +204,10 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // All committed bulk groups have finished reading shared memory.
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// All but the newest committed bulk group have finished reading shared memory.
+__device__ __forceinline__ void bulk_wait_read_but1() {
+  asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+}
 // All committed bulk groups have completed (their global writes are done).
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -279,6 +292,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t (&u)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
+        "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
+      : "r"(taddr)
+      : "memory");
+}
+// 16 rows (the warp's lanes 0..15 of the address, or 16..31) by 32 columns:
+// lane l gets row l / 4 in u[4 j], u[4 j + 1] and row l / 4 + 8 in u[4 j + 2],
+// u[4 j + 3], columns 8 j + 2 (l % 4) and the next, j = 0..3.  No wait (as above).
+__device__ __forceinline__ void tmem_ld16x256_nowait(uint32_t taddr, uint32_t (&u)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]),
         "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15])
       : "r"(taddr)
@@ -448,6 +472,34 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       : "memory");
 }
 
+// Four K16 steps of one 64-deep K block, D (+)= A B, from descriptor halves:
+// warp-collective, one elected lane issues all four.  The low halves advance by
+// sa / sb (>> 4 units) a step; the first step accumulates if `acc` is set.  One
+// election and a handful of adds for four MMAs: the issuing warp shares its
+// scheduler and the instruction cache with busy epilogue warps, and the fewer
+// instructions it needs per MMA, the less it falls behind the tensor core.
+#define SCAL3R_MMA_K64(name, group)                                                                                  \
+  __device__ __forceinline__ void name(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t sa,       \
+                                       uint32_t sb, uint32_t idesc, uint32_t acc) {                                   \
+    asm volatile(                                                                                                     \
+        "{\n\t.reg .pred e, p;\n\t.reg .b64 da, db;\n\t.reg .b32 al, bl;\n\t"                                        \
+        "elect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %7, 0;\n\t"                                                   \
+        "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"                                                         \
+        "@e tcgen05.mma." group ".kind::f16 [%0], da, db, %6, p;\n\t"                                                 \
+        "setp.eq.b32 p, 0, 0;\n\t"                                                                                   \
+        "add.u32 al, %1, %4;\n\tadd.u32 bl, %2, %5;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t"          \
+        "@e tcgen05.mma." group ".kind::f16 [%0], da, db, %6, p;\n\t"                                                 \
+        "add.u32 al, al, %4;\n\tadd.u32 bl, bl, %5;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t"          \
+        "@e tcgen05.mma." group ".kind::f16 [%0], da, db, %6, p;\n\t"                                                 \
+        "add.u32 al, al, %4;\n\tadd.u32 bl, bl, %5;\n\tmov.b64 da, {al, %3};\n\tmov.b64 db, {bl, %3};\n\t"          \
+        "@e tcgen05.mma." group ".kind::f16 [%0], da, db, %6, p;\n\t}" ::"r"(d_tmem),                                 \
+        "r"(a_lo), "r"(b_lo), "r"(hi), "r"(sa), "r"(sb), "r"(idesc), "r"(acc)                                         \
+        : "memory");                                                                                                  \
+  }
+SCAL3R_MMA_K64(mma_k64_w, "cta_group::1")
+SCAL3R_MMA_K64(mma_k64_pair_w, "cta_group::2")
+#undef SCAL3R_MMA_K64
+
 // Arrive on the mbarrier once all previously issued tcgen05 ops of this
 // thread have completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -482,6 +534,70 @@ __device__ __forceinline__ void mma_commit_w(uint64_t* bar) {
   asm volatile(
       "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
       "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
+      : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// CTA pairs (clusters of two on neighbouring SMs, tcgen05 cta_group::2)
+// ---------------------------------------------------------------------------
+// One MMA, issued by the even CTA, multiplies a 256-row A (128 rows in each
+// CTA's shared memory) by a B whose N halves lie in the two CTAs; each CTA's
+// TMEM gets its own 128 rows.  Offsets of operands, barriers and TMEM columns
+// are the same in both CTAs.
+
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// The address of `p` (shared memory of this CTA) in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t mapa_u32(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+// All threads of both CTAs.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+// A tile load into this CTA that completes on a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr,
+                                                 int32_t c0, int32_t c1, int32_t c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr,
+                                                 int32_t c0, int32_t c1, int32_t c2, int32_t c3, int32_t c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      " [%0], [%1, {%3, %4, %5, %6, %7}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
+// One whole warp of each CTA of the pair executes the three of these.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish_pair() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// The commit arrives on the barrier at this offset in both CTAs.
+__device__ __forceinline__ void mma_commit_pair_w(uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+      "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
+          smem_u32(bar)),
+      "h"((uint16_t)3)
       : "memory");
 }
 

@@ -18,14 +18,32 @@
 // pieces (wide_partial_grad, wide_apply_update, wide_apply) and the plain
 // GEMM of the C ABI (wide_gemm_bf16) are built from the same GEMM kernel.
 //
-// All GEMMs run on one persistent tcgen05 kernel: 128 x 256 output tiles, K
-// in steps of 64 through a four-stage TMA pipeline (128-byte swizzle, either
-// operand K- or MN-major), one elected thread of a converged warp issuing
-// M128 N256 K16 MMAs into two 256-column TMEM accumulators in turn, and two
-// groups of four epilogue warps (TMEM lane = output row), one per accumulator.
-// The gate GEMMs read W1 and W3 rows (and -R1, -R3 in the backward) of the same
-// hidden units into one N = 256 operand, so one tile holds every half of the
-// gate.  Epilogues store 32 bytes per thread and row.
+// All GEMMs run on one persistent tcgen05 kernel in two forms: CTA pairs (256 x
+// 256 output tiles on two neighbouring SMs, cta_group::2, each CTA loading its
+// 128 A rows and half of B), or single CTAs (128 x 256) where pairs would need
+// more rounds of tiles (use_pairs).  K advances 64 at a time through a TMA ring
+// (128-byte swizzle, either operand K- or MN-major); a converged warp issues four
+// K16 MMAs a step into two 256-column TMEM accumulators in turn, and eight
+// epilogue warps (TMEM lane = output row) share every tile.  The gate GEMMs read
+// W1 and W3 rows (and -R1, -R3 in the backward) of the same hidden units into one
+// N = 256 operand, so one tile holds every half of the gate.
+//
+// What bounded the single-CTA form, with 52 to 60 % of the tensor pipe active (at
+// head_dim 1024, hidden 4096, 16,656 tokens), and what each change gave:
+//   - operand bytes: 48 KB a K block into an SM that takes in about 57 bytes a
+//     clock; a pair needs 32 KB.  Alone this changed little (P 103 -> 95 us, the
+//     gradient sums 111 -> 114, the gates slower), because of
+//   - the issuing threads: their instructions queue behind busy epilogue warps.
+//     Four MMAs per asm block from descriptor halves, no divisions in the loops:
+//     gradient sums 111 -> 93 us, dk 375 -> 327, inference step 4.17 -> 3.57 ms;
+//     A and B loaded by two warps: gradient sums -> 82 us, dk -> 316.
+//   - the accumulator hand-off: a gate's epilogue took 14,100 cycles a tile on four
+//     warps beside 9,600 of MMAs, and two accumulators then bound a tile at half
+//     the sum; eight warps a tile and gate_tile's stores: apply gate 156 -> 144 us,
+//     gradient gate 205 -> 191 us (225 at first), update-VJP gate 485 -> 447 us.
+// Now the tensor pipe is active 70 to 89 %, the SM clock falls to 1.8 GHz under the
+// power cap, and rounds of tiles (3.47 run as 4) and the gates' stores beside the
+// operand stream are what is left.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -47,7 +65,11 @@ constexpr uint32_t A_STAGE = BM * BK * 2;               // 16 KB
 constexpr uint32_t B_STAGE = BN * BK * 2;               // 32 KB
 constexpr uint32_t STAGE_BYTES = A_STAGE + B_STAGE;
 constexpr size_t GEMM_SMEM = 1024 + STAGES * STAGE_BYTES;
-constexpr int GEMM_THREADS = 320;                       // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue
+constexpr int PAIR_STAGES = 5;                          // CTA pair: a stage is A (16 KB) and half of B (16 KB)
+constexpr uint32_t PAIR_STAGE = A_STAGE + B_STAGE / 2;
+constexpr uint32_t WARP_STAGE = 8192;                   //   and each epilogue warp stages its outputs in 8 KB
+constexpr size_t PAIR_SMEM = 1024 + PAIR_STAGES * PAIR_STAGE + 8 * WARP_STAGE;
+constexpr int GEMM_THREADS = 352;                       // warps 0, 10 TMA, warp 1 MMA, warps 2..9 epilogue
 
 enum Epi : int {
   EPI_F32 = 0,      // out[0] = acc (float32)
@@ -74,6 +96,11 @@ enum Epi : int {
 
 struct GemmArgs {
   CUtensorMap a[4], b[4];  // operand maps: K segment s reads a[s] / b[s]; N block j of the B tile reads b[j]
+  CUtensorMap o[6];        // CTA pairs: output maps (staged epilogues), see staged_epi
+  const void* bw[2];       // gate products: the weight matrices [b_rows][K] behind b[] (host side)
+  int64_t b_rows;
+  int gated;               // CTA pairs: b[] permutes the hidden units for gate_tile
+  int staged;              // CTA pairs: the update-VJP gate's outputs are staged
   int M, N, K;             // output rows, output columns (N = 256 * tiles), reduction length
   int kseg, nseg;          // nseg > 1: K is nseg segments of kseg (a multiple of 64)
   int nbn;                 // > 1: the B tile is nbn blocks of 256 / nbn rows (K-major, one segment)
@@ -213,29 +240,413 @@ __device__ __forceinline__ void store_deta(const GemmArgs& g, int m, int tn, flo
   }
 }
 
-template <bool XSET>
+// Staged epilogues (CTA pairs).  TMEM lane = output row, so a direct store of a
+// warp touches 32 rows.  Instead each warp writes its 32 rows of a column group
+// (128-byte rows: 64 bf16 or 32 float32 columns) to its own 8 KB of shared
+// memory (two groups), in the 128-byte swizzle (conflict-free 16-byte stores),
+// and one lane sends the group off with TMA; the map clips the rows past M.  The
+// accumulating epilogue is a TMA add.
+struct OutStage {
+  uint8_t* buf;
+  int lane;
+  // 16-byte chunk c of this lane's row of the group at byte b
+  __device__ __forceinline__ void put(int b, int c, const uint4& v) const {
+    *reinterpret_cast<uint4*>(buf + b + lane * 128 + ((c ^ (lane & 7)) << 4)) = v;
+  }
+  // chunk c (0 or 1) of this lane's 32-byte row
+  __device__ __forceinline__ void put32(int b, int c, const uint4& v) const {
+    *reinterpret_cast<uint4*>(buf + b + lane * 32 + ((c ^ ((lane >> 2) & 1)) << 4)) = v;
+  }
+  // the buffers are free once TMA has read them: all groups, or all but the newest
+  __device__ __forceinline__ void reuse(bool keep1) const {
+    if (lane == 0) {
+      if (keep1) bulk_wait_read_but1();
+      else bulk_wait_read_all();
+    }
+    __syncwarp();
+  }
+  // every lane's writes visible to TMA; lane 0 then stores
+  __device__ __forceinline__ bool ready() const {
+    fence_proxy_async_smem();
+    __syncwarp();
+    return lane == 0;
+  }
+};
+
+__device__ __forceinline__ uint4 pack8f(const float* v) {
+  return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+}
+
+// 32 accumulator columns of this lane's row, in two halves.
+__device__ __forceinline__ void tmem_ld32(uint32_t a, float (&v)[32]) {
+  uint32_t u0[16], u1[16];
+  tmem_ld16_nowait(a, u0);
+  tmem_ld16_nowait(a + 16, u1);
+  tmem_wait_ld16(u0);
+  tmem_wait_ld16(u1);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    v[i] = __uint_as_float(u0[i]);
+    v[16 + i] = __uint_as_float(u1[i]);
+  }
+}
+
+// The chain rule of the update-VJP gate on eight hidden units of one row:
+// z1, z3, dg1, dg3 in zz, p = W2^T v, n = -R2^T v, the negated rates n1, n3, n2;
+// eight bf16 of each output into o, the d eta partials (negated) added to aq.
+__device__ __forceinline__ void bkey8(const float (&zz)[4][8], const uint4& pw, const uint4& nw, float e1, float e3,
+                                      float e2, uint32_t (&o)[6][4], f32x2 (&aq)[3]) {
+  float praw[8], ndu[8];
+  unpack8(pw, praw);
+  unpack8(nw, ndu);
+  const f32x2 n1 = x2(-e1), n3 = x2(-e3), n2 = x2(-e2), one = x2(1.f), two = x2(2.f), mtwo = x2(-2.f);
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const int e = 2 * w;
+    const f32x2 x1 = x2(zz[0][e], zz[0][e + 1]), x3 = x2(zz[1][e], zz[1][e + 1]);
+    const f32x2 d1 = x2(zz[2][e], zz[2][e + 1]), d3 = x2(zz[3][e], zz[3][e + 1]);
+    const f32x2 pr = x2(praw[e], praw[e + 1]), nd = x2(ndu[e], ndu[e + 1]);
+    const f32x2 sg = sigmoid2(x1);
+    const f32x2 a = mul2(x1, sg);
+    const f32x2 oms = sub2(one, sg);
+    const f32x2 sp = fma2(a, oms, sg);                                         // silu'(z1)
+    const f32x2 spp = mul2(mul2(sg, oms), fma2(x1, fma2(mtwo, sg, one), two));  // silu''(z1)
+    const f32x2 u = mul2(a, x3);
+    const f32x2 p1 = mul2(n1, pr), p3 = mul2(n3, pr);   // rate times p (e = -v)
+    const f32x2 du = mul2(n2, nd);
+    const f32x2 x3sp = mul2(x3, sp);
+    const f32x2 t1 = mul2(d1, x3sp);
+    const f32x2 d3a = mul2(d3, a);
+    const f32x2 da = fma2(d3, p3, mul2(du, x3));
+    const f32x2 dp1 = mul2(d1, p1);
+    o[1][w] = pack_bf16x2(fma2(dp1, sp, mul2(du, a)));                 // dz3
+    o[0][w] = pack_bf16x2(fma2(mul2(dp1, x3), spp, mul2(da, sp)));     // dz1
+    o[2][w] = pack_bf16x2(mul2(p1, x3sp));                           // g1
+    o[3][w] = pack_bf16x2(mul2(p3, a));                              // g3
+    o[4][w] = pack_bf16x2(fma2(n1, t1, mul2(n3, d3a)));              // -dp
+    o[5][w] = pack_bf16x2(mul2(n2, u));                              // -eta2 u
+    aq[0] = fma2(pr, t1, aq[0]);
+    aq[1] = fma2(pr, d3a, aq[1]);
+    aq[2] = fma2(nd, u, aq[2]);
+  }
+}
+
+// The gradient / apply-VJP gate on eight hidden units of one row: r = W2^T v,
+// W2^T e or W2^T d_o; scales s1, s3, s2 -> g1, g3, u~ (or dzq1, dzq3, uq).
+__device__ __forceinline__ void gate8(const float* z1, const float* z3, const uint4& rw, f32x2 s1, f32x2 s3, f32x2 s2,
+                                      uint32_t (&o)[3][4]) {
+  float r[8];
+  unpack8(rw, r);
+  const f32x2 one = x2(1.f);
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const f32x2 x1 = x2(z1[2 * w], z1[2 * w + 1]), x3 = x2(z3[2 * w], z3[2 * w + 1]);
+    const f32x2 rr = x2(r[2 * w], r[2 * w + 1]);
+    const f32x2 sg = sigmoid2(x1);
+    const f32x2 a = mul2(x1, sg);
+    const f32x2 sp = fma2(a, sub2(one, sg), sg);        // silu'(z1)
+    o[0][w] = pack_bf16x2(mul2(mul2(mul2(s1, rr), x3), sp));
+    o[1][w] = pack_bf16x2(mul2(mul2(s3, rr), a));
+    o[2][w] = pack_bf16x2(mul2(s2, mul2(a, x3)));
+  }
+}
+
+// A 16-byte store of eight bf16.
+__device__ __forceinline__ void st16(__nv_bfloat16* p, const uint32_t (&w)[4]) {
+  if (in_bounds(p, 16)) *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Gate epilogues of CTA pairs.  With a row per lane, each store of a warp
+// touches 32 rows and each load of an input fetches 16 bytes of 32 lines: those
+// transactions, not the arithmetic, kept the accumulators from the MMAs.  TMEM
+// loads of 16 rows x 32 columns give a lane two columns of every eight, four
+// lanes a row; the map of the weights (gate_map) orders the hidden units so that
+// a lane's eight columns of a 32-column group are eight consecutive hidden units
+// (TMEM column 8 j + 2 t + p of a group holds hidden unit 8 t + 2 j + p).  So a
+// lane loads and stores 16 bytes, four lanes 64 contiguous bytes of a row, from
+// registers, and the TMA engine (57 bytes a clock and SM measured, just what the
+// operand loads take) carries no outputs.  Lane l owns rows row0 + l / 4 + 8 k;
+// gp: the half of the tile's hidden units.
+__device__ __forceinline__ void gate_tile(const GemmArgs& g, uint32_t acc, int lane, int row0, int tn, int gp) {
+  const int t8 = 8 * (lane & 3), r0 = row0 + (lane >> 2);
+  const int f0 = tn * (BN / 2);
+  const int64_t ld = g.ld_out;
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+  // z1 | z3 of 128 hidden units: KEY (in0 = W2^T v or W2^T e), BAPPLY (in0 = W2^T d_o) or APPLY
+  const bool key = g.epi == EPI_KEY, apply = g.epi == EPI_APPLY;
+  f32x2 s1[4], s3[4], s2[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float e1 = 0.f, e3 = 0.f, e2 = 0.f;
+    if (key && r0 + 8 * k < g.M) row_rates(g, r0 + 8 * k, e1, e3, e2);
+    if (!g.mse) {   // dot loss: e = -eta v
+      e1 = -e1;
+      e3 = -e3;
+    }
+    s1[k] = x2(key ? e1 : 1.f);
+    s3[k] = x2(key ? e3 : 1.f);
+    s2[k] = x2(key ? -e2 : 1.f);
+  }
+  // two row halves in turn: one half's TMEM and input loads are in flight while
+  // the other half is computed
+  uint32_t z1[2][16], z3[2][16];
+  uint4 pw[2][2];
+  auto fetch = [&](int c, int hs, uint32_t (&a)[16], uint32_t (&b)[16], uint4 (&w)[2]) {
+    tmem_ld16x256_nowait(acc + (hs << 20) + c, a);
+    tmem_ld16x256_nowait(acc + (hs << 20) + 128 + c, b);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = r0 + 16 * hs + 8 * i;
+      w[i] = (!apply && r < g.M) ? ldg16(reinterpret_cast<const uint4*>(g.in0 + (size_t)r * ld + f0 + c + t8)) : zero;
+    }
+  };
+  auto compute = [&](int c, int hs, uint32_t (&a)[16], uint32_t (&b)[16], uint4 (&w)[2]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int k = 2 * hs + i, r = r0 + 8 * k;
+      float x1[8], x3[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        x1[j] = __uint_as_float(a[4 * (j >> 1) + 2 * i + (j & 1)]);
+        x3[j] = __uint_as_float(b[4 * (j >> 1) + 2 * i + (j & 1)]);
+      }
+      const size_t off = (size_t)r * ld + f0 + c + t8;
+      if (apply) {
+        uint32_t hw[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const f32x2 x = x2(x1[2 * j], x1[2 * j + 1]);
+          hw[j] = pack_bf16x2(mul2(mul2(x, sigmoid2(x)), x2(x3[2 * j], x3[2 * j + 1])));
+        }
+        if (r < g.M) st16(reinterpret_cast<__nv_bfloat16*>(g.out[0]) + off, hw);
+      } else {
+        uint32_t o[3][4];
+        gate8(x1, x3, w[i], s1[k], s3[k], s2[k], o);
+        if (r < g.M) {
+          st16(reinterpret_cast<__nv_bfloat16*>(g.out[0]) + off, o[0]);
+          st16(reinterpret_cast<__nv_bfloat16*>(g.out[1]) + off, o[1]);
+          if (g.out[2]) st16(reinterpret_cast<__nv_bfloat16*>(g.out[2]) + off, o[2]);
+        }
+      }
+    }
+  };
+  const int cb = gp * (BN / 4), ce = cb + BN / 4;
+  fetch(cb, 0, z1[0], z3[0], pw[0]);
+#pragma unroll 1
+  for (int c = cb; c < ce; c += 32) {
+    tmem_wait_ld16(z1[0]);
+    tmem_wait_ld16(z3[0]);
+    fetch(c, 1, z1[1], z3[1], pw[1]);
+    compute(c, 0, z1[0], z3[0], pw[0]);
+    tmem_wait_ld16(z1[1]);
+    tmem_wait_ld16(z3[1]);
+    if (c + 32 < ce) fetch(c + 32, 0, z1[0], z3[0], pw[0]);
+    compute(c, 1, z1[1], z3[1], pw[1]);
+  }
+}
+
+// The update-VJP gate's tile: z1 | z3 | dg1 | dg3 of 64 hidden units, a row per
+// lane, six outputs of 16 columns at a time (32-byte rows, 1 KB each).  A row's d
+// eta partial is one chain over the tile's hidden units (the order of the
+// direct epilogue), so one warp takes all of a row's columns.
+__device__ __forceinline__ void staged_bkey(const GemmArgs& g, const OutStage& st, uint32_t acc, int m, int tn) {
+  const int row0 = m - st.lane;
+  const bool valid = m < g.M;
+  const bool any = row0 < g.M;   // the warp has rows to store
+  const int f0 = tn * (BN / 4);
+  float e1 = 0.f, e3 = 0.f, e2 = 0.f;
+  if (valid) row_rates(g, m, e1, e3, e2);
+  f32x2 aq[3] = {x2(0.f), x2(0.f), x2(0.f)};
+  const uint4* pp = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * g.ld_out + f0);
+  const uint4* np = reinterpret_cast<const uint4*>(g.in1 + (size_t)m * g.ld_out + f0);
+  const uint4 zero = make_uint4(0, 0, 0, 0);
+  uint4 pw[2], nw[2];   // the inputs of 16 columns, one group ahead
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    pw[j] = valid ? ldg16(pp + j) : zero;
+    nw[j] = valid ? ldg16(np + j) : zero;
+  }
+#pragma unroll 1
+  for (int c = 0; c < 64; c += 16) {
+    uint4 pn[2] = {zero, zero}, nn[2] = {zero, zero};
+    if (c + 16 < 64 && valid) {
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        pn[j] = ldg16(pp + c / 8 + 2 + j);
+        nn[j] = ldg16(np + c / 8 + 2 + j);
+      }
+    }
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const int cc = c + 8 * hh;
+      float zz[4][8];
+      tmem_ld8x4(acc + cc, acc + 64 + cc, acc + 128 + cc, acc + 192 + cc, zz);
+      uint32_t o[6][4];
+      bkey8(zz, pw[hh], nw[hh], e1, e3, e2, o, aq);
+      if (hh == 0) st.reuse(false);
+#pragma unroll
+      for (int q = 0; q < 6; ++q) st.put32(1024 * q, hh, make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]));
+    }
+    if (st.ready() && any) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) tma_store_3d(&g.o[q], st.buf + 1024 * q, f0 + c, row0, 0);
+      bulk_commit();
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      pw[j] = pn[j];
+      nw[j] = nn[j];
+    }
+  }
+  if (valid)
+    store_deta(g, m, tn, -(x2_lo(aq[0]) + x2_hi(aq[0])), -(x2_lo(aq[1]) + x2_hi(aq[1])),
+               -(x2_lo(aq[2]) + x2_hi(aq[2])));
+}
+
+// One tile's staged epilogue: accumulator columns acc + cb .. acc + cb + 127 of
+// this warp's 32 lanes, output rows m - lane .. (m: this lane's), columns n0 + cb
+// ..; plane: the K range's partial plane.
+__device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& st, uint32_t acc, int m, int n0, int cb,
+                                            int plane) {
+  const int row0 = m - st.lane;
+  const bool valid = m < g.M;
+  const bool any = row0 < g.M;   // the warp has rows to store
+  if (g.epi == EPI_F32 || g.epi == EPI_F32_ADD || g.epi == EPI_F32_ADDIN) {
+    const uint4* xin = nullptr;
+    if (g.epi == EPI_F32_ADDIN)
+      xin = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * (g.ld_in ? g.ld_in : g.ld_out) + n0);
+#pragma unroll 2
+    for (int c = cb; c < cb + BN / 2; c += 32) {
+      uint4 xw[4];
+      if (xin) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xw[j] = valid ? ldg16(xin + c / 8 + j) : make_uint4(0, 0, 0, 0);
+      }
+      float v[32];
+      tmem_ld32(acc + c, v);
+      if (xin) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float x[8];
+          unpack8(xw[j], x);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[8 * j + i] += x[i];
+        }
+      }
+      const int b = ((c >> 5) & 1) * 4096;
+      st.reuse(true);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        st.put(b, j, make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]),
+                                   __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3])));
+      if (st.ready() && any) {
+        if (g.epi == EPI_F32_ADD) tma_reduce_add_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
+        else tma_store_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
+        bulk_commit();
+      }
+    }
+    return;
+  }
+  if (g.epi == EPI_GCM_GATE) {
+    const uint4* xin = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * (g.ld_in ? g.ld_in : g.ld_out) + n0);
+#pragma unroll 1
+    for (int c0 = cb; c0 < cb + BN / 2; c0 += 64) {
+      uint4 xw[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) xw[j] = valid ? ldg16(xin + c0 / 8 + j) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int hh = 0; hh < 2; ++hh) {
+        float v[32];
+        tmem_ld32(acc + c0 + 32 * hh, v);
+        if (hh == 0) st.reuse(false);
+        const float* al = g.colvec + n0 + c0 + 32 * hh;
+        const bool okc = in_bounds(al, 128);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          st.put(4096, 4 * hh + j, pack8f(v + 8 * j));   // y
+          float x[8];
+          unpack8(xw[4 * hh + j], x);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[i] = fmaf(okc ? al[8 * j + i] : 0.f, v[8 * j + i], x[i]);
+          st.put(0, 4 * hh + j, pack8f(x));
+        }
+      }
+      if (st.ready() && any) {
+        tma_store_3d(&g.o[0], st.buf, n0 + c0, row0, 0);
+        tma_store_3d(&g.o[1], st.buf + 4096, n0 + c0, row0, 0);
+        bulk_commit();
+      }
+    }
+    return;
+  }
+  // one bf16 output: the product, or one of q, k, v
+  const bool qkv = g.epi == EPI_GCM_QKV;
+  const int dm = (int)g.ld_out, part = qkv ? n0 / dm : 0;   // qkv: the tile's columns lie in one of q, k, v
+  const int oc = n0 - part * dm;
+#pragma unroll 1
+  for (int c0 = cb; c0 < cb + BN / 2; c0 += 64) {
+    const int b = ((c0 >> 6) & 1) * 4096;
+    float ss = 0.f;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const int c = c0 + 32 * hh;
+      float v[32];
+      tmem_ld32(acc + c, v);
+      if (qkv) {
+        const float* bb = g.colvec + n0 + c;
+        if (in_bounds(bb, 128)) {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] += bb[i];
+        }
+        if (part < 2) {   // the norm from the float32 values, in the order of the direct epilogue
+#pragma unroll
+          for (int i = 0; i < 16; ++i) ss = fmaf(v[16 + i], v[16 + i], fmaf(v[i], v[i], ss));
+        }
+      }
+      if (hh == 0) st.reuse(true);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) st.put(b, 4 * hh + j, pack8f(v + 8 * j));
+    }
+    if (qkv && part < 2 && valid) {
+      float* ssq = reinterpret_cast<float*>(g.out[3]) + (size_t)m * g.ld_part + (part * dm + oc + c0) / 64;
+      if (in_bounds(ssq, 4)) *ssq = ss;
+    }
+    if (st.ready() && any) {
+      tma_store_3d(&g.o[part], st.buf + b, oc + c0, row0, 0);
+      bulk_commit();
+    }
+  }
+}
+
+template <bool XSET, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid_constant__ GemmArgs g) {
+  constexpr int NST = PAIR ? PAIR_STAGES : STAGES;
+  constexpr uint32_t STG = PAIR ? PAIR_STAGE : STAGE_BYTES;
+  constexpr int TM = PAIR ? 2 * BM : BM;                 // rows of a tile (the pair's)
+  constexpr bool SHARE = !XSET;                          // both epilogue groups work on every tile
   extern __shared__ uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], never_bar;
+  __shared__ uint64_t full[NST], empty[NST], acc_full[2], acc_empty[2], never_bar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int tiles_n = g.N / BN;
-  const int ntiles = ((g.M + BM - 1) / BM) * tiles_n;
+  const int ntiles = ((g.M + TM - 1) / TM) * tiles_n;
   const int nunits = ntiles * g.ksplit;   // work units: K range s of tile t is unit s * ntiles + t
+  const int rank = PAIR ? (int)cluster_ctarank() : 0;    // rows [128 rank, 128 rank + 128) of a pair's tile
+  const int u0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, ustep = PAIR ? gridDim.x >> 1 : gridDim.x;
   const int nk = (g.K + BK - 1) / BK;
   const int kps = g.nseg > 1 ? g.kseg / BK : nk;   // K blocks per segment
   volatile int* abort = &abort_flag;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < NST; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 4);
+      mbar_init(&acc_empty[i], (PAIR ? 2 : 1) * (SHARE ? 8 : 4));   // a tile's epilogue warps (of both CTAs)
     }
     mbar_init(&never_bar, 1);   // no thread ever arrives
     abort_flag = 0;
@@ -244,116 +655,182 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
     for (int j = 0; j < (g.nbn > g.nseg ? g.nbn : g.nseg); ++j) prefetch_tmap(&g.b[j]);
   }
   if (warp == 1) {
-    tmem_alloc(&tmem_base, 512);
-    tmem_relinquish();
+    if (PAIR) {
+      tmem_alloc_pair(&tmem_base, 512);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(&tmem_base, 512);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync();   // the other CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tb = tmem_base;
 
-  if (warp == 0) {
+  if (warp == 0 || warp == 10) {
+    // producers: one thread of warp 0 loads A, one of warp 10 loads B (a lone
+    // thread took 460 to 550 cycles for a stage's three or four loads, as long
+    // as the stage's MMAs).  Each CTA of a pair loads its own A rows and its
+    // half of B; all loads of a stage complete on the even CTA's barrier.
     if (lane == 0) {
-      uint32_t it = 0;
+      const bool is_a = warp == 0;
+      int s = 0;
+      uint32_t ph = 1;   // the parity that frees stage s
       bool ok = true;
-      for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
+      const uint32_t lead_full = PAIR ? mapa_u32(&full[0], 0) : 0u;
+      const int nb = PAIR ? g.nbn / 2 : g.nbn, brows = BN / g.nbn;   // N blocks of this CTA's B, and their rows
+      const uint32_t bblk = B_STAGE / g.nbn;
+      for (int u = u0; u < nunits && ok; u += ustep) {
         const int t = u % ntiles, ks0 = (u / ntiles) * g.kb_split;
         const int tm = t / tiles_n, tn = t % tiles_n;
-        const int m0 = tm * BM, n0 = tn * BN;
+        const int m0 = tm * TM + rank * BM, n0 = tn * BN + rank * (BN / 2);
         const int kb_end = min(nk, ks0 + g.kb_split);
-        for (int kb = ks0; kb < kb_end; ++kb, ++it) {
-          const int s = it % STAGES;
-          if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1, abort)) {
+        int sg = ks0 / kps, k0 = (ks0 % kps) * BK;   // K segment and the block's place in it
+        for (int kb = ks0; kb < kb_end; ++kb) {
+          if (!mbar_wait(&empty[s], ph, abort)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-          uint8_t* as = sm + s * STAGE_BYTES;
+          const uint32_t lf = lead_full + 8 * s;
+          auto load = [&](void* dst, const CUtensorMap* map, int c0, int c1, int c2) {
+            if (PAIR) tma_load_3d_pair(dst, map, lf, c0, c1, c2);
+            else tma_load_3d(dst, map, &full[s], c0, c1, c2);
+          };
+          uint8_t* as = sm + s * STG;
           uint8_t* bs = as + A_STAGE;
-          const int sg = kb / kps, k0 = (kb % kps) * BK;
-          const CUtensorMap* am = &g.a[sg];
-          if (!g.a_mn) {
-            tma_load_3d(as, am, &full[s], k0, g.ha, g.ya + m0);
-          } else {
-            tma_load_3d(as, am, &full[s], m0, g.ha, g.ya + k0);
-            tma_load_3d(as + 8192, am, &full[s], m0 + 64, g.ha, g.ya + k0);
-          }
-          if (g.nbn > 1) {
-            const int rows = BN / g.nbn;
-            for (int j = 0; j < g.nbn; ++j)
-              tma_load_3d(bs + j * (B_STAGE / g.nbn), &g.b[j], &full[s], k0, g.hb, g.yb + tn * rows);
+          if (is_a) {
+            if (rank == 0) mbar_arrive_expect_tx(&full[s], PAIR ? 2 * STG : STG);   // A's and B's bytes
+            const CUtensorMap* am = &g.a[sg];
+            if (!g.a_mn) {
+              load(as, am, k0, g.ha, g.ya + m0);
+            } else {
+              load(as, am, m0, g.ha, g.ya + k0);
+              load(as + 8192, am, m0 + 64, g.ha, g.ya + k0);
+            }
+          } else if (g.nbn > 1) {
+            for (int j = 0; j < nb; ++j) {
+              if (PAIR && g.gated)
+                tma_load_5d_pair(bs + j * bblk, &g.b[rank * nb + j], lf, k0, 0, 0, 0, tn * brows / 32);
+              else
+                load(bs + j * bblk, &g.b[rank * nb + j], k0, g.hb, g.yb + tn * brows);
+            }
           } else if (!g.b_mn) {
-            tma_load_3d(bs, &g.b[sg], &full[s], k0, g.hb, g.yb + n0);
+            load(bs, &g.b[sg], k0, g.hb, g.yb + n0);
+            if (!PAIR) load(bs + B_STAGE / 2, &g.b[sg], k0, g.hb, g.yb + n0 + BN / 2);
           } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) tma_load_3d(bs + 8192 * j, &g.b[sg], &full[s], n0 + 64 * j, g.hb, g.yb + k0);
+            for (int j = 0; j < (PAIR ? 2 : 4); ++j) load(bs + 8192 * j, &g.b[sg], n0 + 64 * j, g.hb, g.yb + k0);
+          }
+          if (++s == NST) {
+            s = 0;
+            ph ^= 1;
+          }
+          k0 += BK;
+          if (k0 == kps * BK) {
+            k0 = 0;
+            ++sg;
           }
         }
       }
+      // the pair's last stage releases have arrived before this CTA ends
+      if (PAIR)
+        for (int k = 0; k < NST && ok; ++k) {
+          ok = mbar_wait(&empty[s], ph, abort);
+          if (++s == NST) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
     }
     __syncwarp();
   } else if (warp == 1) {
-    const uint32_t idesc = idesc_bf16(BM, BN, g.a_mn != 0, g.b_mn != 0);
-    uint32_t it = 0;
-    int i = 0;
-    bool ok = true;
-    for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++i) {
+    const uint32_t idesc = idesc_bf16(TM, BN, g.a_mn != 0, g.b_mn != 0);
+    const uint32_t a0 = sdesc_lo(smem_u32(sm), g.a_mn ? 8192 : 16);
+    const uint32_t b0 = sdesc_lo(smem_u32(sm) + A_STAGE, g.b_mn ? 8192 : 16);
+    const uint32_t sa = (g.a_mn ? 2048 : 32) >> 4, sb = (g.b_mn ? 2048 : 32) >> 4;   // a K16 step
+    constexpr uint32_t HI = sdesc_hi(1024, kSwizzle128);
+    int s = 0, i = 0;
+    uint32_t ph = 0;
+    bool ok = rank == 0;   // the even CTA issues for the pair
+    for (int u = u0; u < nunits && ok; u += ustep, ++i) {
       const int ac = i & 1;
       const int ks0 = (u / ntiles) * g.kb_split, kb_end = min(nk, ks0 + g.kb_split);
       if (!mbar_wait_w(&acc_empty[ac], ((i >> 1) & 1) ^ 1, abort)) break;
       tc_fence_after();
       const uint32_t acc = tb + ac * 256;
-      for (int kb = ks0; kb < kb_end; ++kb, ++it) {
-        const int s = it % STAGES;
-        if (!mbar_wait_w(&full[s], (it / STAGES) & 1, abort)) {
+      uint32_t add = 0;
+      for (int kb = ks0; kb < kb_end; ++kb) {
+        if (!mbar_wait_w(&full[s], ph, abort)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t as = smem_u32(sm + s * STAGE_BYTES), bs = as + A_STAGE;
-#pragma unroll
-        for (int ks = 0; ks < BK / 16; ++ks) {
-          const uint64_t ad = g.a_mn ? sdesc_sw128(as + ks * 2048, 8192, 1024) : sdesc_sw128(as + ks * 32, 16, 1024);
-          const uint64_t bd = g.b_mn ? sdesc_sw128(bs + ks * 2048, 8192, 1024) : sdesc_sw128(bs + ks * 32, 16, 1024);
-          mma_ss_w(acc, ad, bd, idesc, (kb > ks0 || ks > 0) ? 1u : 0u);
+        const uint32_t off = s * (STG >> 4);
+        if (PAIR) {
+          mma_k64_pair_w(acc, a0 + off, b0 + off, HI, sa, sb, idesc, add);
+          mma_commit_pair_w(&empty[s]);
+        } else {
+          mma_k64_w(acc, a0 + off, b0 + off, HI, sa, sb, idesc, add);
+          mma_commit_w(&empty[s]);
         }
-        mma_commit_w(&empty[s]);
+        add = 1;
+        if (++s == NST) {
+          s = 0;
+          ph ^= 1;
+        }
       }
-      if (ok) mma_commit_w(&acc_full[ac]);
+      if (ok) {
+        if (PAIR) mma_commit_pair_w(&acc_full[ac]);
+        else mma_commit_w(&acc_full[ac]);
+      }
     }
   } else {
-    // epilogue group gp = warps 2..5 (gp 0) or 6..9 (gp 1); thread = output
-    // row m0 + row of the TMEM lanes of this warp
+    // epilogue: thread = output row m0 + row of the TMEM lanes of this warp.
+    // SHARE: warps 2..5 (gp 0) and 6..9 (gp 1) take half of every tile's columns
+    // each.  (A tile per group leaves a tile's accumulator twice as long in the
+    // epilogue; with two accumulators the MMAs then wait whenever the epilogue
+    // of a tile takes longer than the MMAs of the next, as the gates' does.)
+    // Else group gp takes the tiles of accumulator gp.
     const int gp = (warp - 2) >> 2;
     const uint32_t row = 32u * (warp & 3) + lane;
     const uint32_t lane_base = (32u * (warp & 3)) << 16;
-    const uint32_t accb = tb + lane_base + gp * 256;
-    int i = gp;
-    for (int u = blockIdx.x + gp * gridDim.x; u < nunits; u += 2 * gridDim.x, i += 2) {
+    const uint32_t lead_empty = PAIR ? mapa_u32(&acc_empty[0], 0) : 0u;
+    constexpr int IS = SHARE ? 1 : 2;
+    int i = SHARE ? 0 : gp;
+    for (int u = u0 + i * ustep; u < nunits; u += IS * ustep, i += IS) {
+      const uint32_t accb = tb + lane_base + (i & 1) * 256;
       if (!XSET && (g.epi == EPI_GCM_GATE || g.epi == EPI_F32_ADDIN)) {
-        // the row's addend (x, or the residual gradient) of this group's next
-        // tile (and of its first) into L2 while products finish: the column
-        // loop below then waits on L2, not HBM
-        for (int up = (i == gp ? u : u + 2 * (int)gridDim.x); up <= u + 2 * (int)gridDim.x && up < nunits;
-             up += 2 * (int)gridDim.x) {
+        // the row's addend (x, or the residual gradient) of this warp's half of
+        // the next tile (and of its first) into L2 while products finish: the
+        // column loop below then waits on L2, not HBM
+        for (int up = (i == 0 ? u : u + ustep); up <= u + ustep && up < nunits; up += ustep) {
           const int tp = up % ntiles;
-          const int mp = (tp / tiles_n) * BM + (int)row, np = (tp % tiles_n) * BN;
+          const int mp = (tp / tiles_n) * TM + rank * BM + (int)row, np = (tp % tiles_n) * BN + gp * (BN / 2);
           if (mp < g.M) {
             const __nv_bfloat16* src = g.in0 + (size_t)mp * (g.ld_in ? g.ld_in : g.ld_out) + np;
-            if (in_bounds(src, BN * 2)) bulk_prefetch_l2(src, BN * 2);
+            if (in_bounds(src, BN)) bulk_prefetch_l2(src, BN);
           }
         }
       }
-      if (!mbar_wait(&acc_full[gp], (i >> 1) & 1, abort)) break;
+      if (!mbar_wait(&acc_full[i & 1], (i >> 1) & 1, abort)) break;
       tc_fence_after();
       const int t = u % ntiles;
       float* const part_plane = g.ksplit > 1 ? reinterpret_cast<float*>(g.out[0]) + (u / ntiles) * g.split_stride
                                              : reinterpret_cast<float*>(g.out[0]);
       const int tm = t / tiles_n, tn = t % tiles_n;
-      const int m0 = tm * BM, n0 = tn * BN;
+      const int m0 = tm * TM + rank * BM, n0 = tn * BN;
       const int m = m0 + (int)row;
       const bool valid = m < g.M;
-      if (XSET && g.epi != EPI_BKEY) {
+      const OutStage ost{sm + NST * STG + (warp - 2) * WARP_STAGE, lane};
+      if (PAIR && !XSET && g.gated) {
+        gate_tile(g, accb, lane, m0 + 32 * (warp & 3), tn, gp);
+      } else if (PAIR && !XSET) {   // every epilogue of the common pair kernel is gated or staged
+        staged_tile(g, ost, accb, m, n0, gp * (BN / 2), u / ntiles);
+      } else if (PAIR && XSET && g.staged) {
+        staged_bkey(g, ost, accb, m, tn);
+      } else if (XSET && g.epi != EPI_BKEY) {
         float e1 = 0.f, e3 = 0.f, e2 = 0.f;
         if (g.eta && valid) row_rates(g, m, e1, e3, e2);
         if (g.epi == EPI_MSE_E || g.epi == EPI_ADD_BF16 || g.epi == EPI_MSE_DE) {
@@ -473,7 +950,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
         }
       } else if (!XSET && (g.epi == EPI_F32 || g.epi == EPI_BF16 || g.epi == EPI_F32_ADD)) {
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = gp * (BN / 2); c < (gp + 1) * (BN / 2); c += 32) {
           float v0[16], v1[16];
           tmem_ld16(accb + c, v0);
           tmem_ld16(accb + c + 16, v1);
@@ -506,7 +983,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
         float* ssq = reinterpret_cast<float*>(g.out[3]) + (size_t)m * g.ld_part + (part * dm + c0) / 64;
         float ss = 0.f;
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = gp * (BN / 2); c < (gp + 1) * (BN / 2); c += 32) {
           float v0[16], v1[16];
           tmem_ld16(accb + c, v0);
           tmem_ld16(accb + c + 16, v1);
@@ -534,7 +1011,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
         // the addend in batches of 64 columns: eight 16-byte loads in flight
         // per thread, so a tile waits four memory round trips, not eight
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 64) {
+        for (int c0 = gp * (BN / 2); c0 < (gp + 1) * (BN / 2); c0 += 64) {
           const uint4* xin = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * ldi + n0 + c0);
           const bool okx = valid && in_bounds(xin, 128);
           uint4 xw[8];
@@ -592,7 +1069,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
         const int f0 = tn * (BN / 4);
         float e1 = 0.f, e3 = 0.f, e2 = 0.f;
         if (valid) row_rates(g, m, e1, e3, e2);
-        f32x2 aq1 = x2(0.f), aq3 = x2(0.f), aq2 = x2(0.f);   // d eta partials, negated, per lane
+        f32x2 aq[3] = {x2(0.f), x2(0.f), x2(0.f)};   // d eta partials, negated, per lane
         const uint4* pp = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * g.ld_out + f0);
         const uint4* np = reinterpret_cast<const uint4*>(g.in1 + (size_t)m * g.ld_out + f0);
 #pragma unroll 1
@@ -609,40 +1086,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
             const int cc = c + 8 * hh;
             float zz[4][8];
             tmem_ld8x4(accb + cc, accb + 64 + cc, accb + 128 + cc, accb + 192 + cc, zz);
-            float praw[8], ndu[8];
-            unpack8(pcur[hh], praw);
-            unpack8(ncur[hh], ndu);
-            // the chain rule on pairs of hidden units (packed float32 lanes)
-            const f32x2 n1 = x2(-e1), n3 = x2(-e3), n2 = x2(-e2), one = x2(1.f), two = x2(2.f), mtwo = x2(-2.f);
+            uint32_t o[6][4];
+            bkey8(zz, pcur[hh], ncur[hh], e1, e3, e2, o, aq);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-              const int e = 2 * w;
-              const f32x2 x1 = x2(zz[0][e], zz[0][e + 1]), x3 = x2(zz[1][e], zz[1][e + 1]);
-              const f32x2 d1 = x2(zz[2][e], zz[2][e + 1]), d3 = x2(zz[3][e], zz[3][e + 1]);
-              const f32x2 pr = x2(praw[e], praw[e + 1]), nd = x2(ndu[e], ndu[e + 1]);
-              const f32x2 sg = sigmoid2(x1);
-              const f32x2 a = mul2(x1, sg);
-              const f32x2 oms = sub2(one, sg);
-              const f32x2 sp = fma2(a, oms, sg);                                         // silu'(z1)
-              const f32x2 spp = mul2(mul2(sg, oms), fma2(x1, fma2(mtwo, sg, one), two));  // silu''(z1)
-              const f32x2 u = mul2(a, x3);
-              const f32x2 p1 = mul2(n1, pr), p3 = mul2(n3, pr);   // rate times p (e = -v)
-              const f32x2 du = mul2(n2, nd);
-              const f32x2 x3sp = mul2(x3, sp);
-              const f32x2 t1 = mul2(d1, x3sp);
-              const f32x2 d3a = mul2(d3, a);
-              const f32x2 da = fma2(d3, p3, mul2(du, x3));
-              const f32x2 dp1 = mul2(d1, p1);
-              pk[1][4 * hh + w] = pack_bf16x2(fma2(dp1, sp, mul2(du, a)));                 // dz3
-              pk[0][4 * hh + w] = pack_bf16x2(fma2(mul2(dp1, x3), spp, mul2(da, sp)));     // dz1
-              pk[2][4 * hh + w] = pack_bf16x2(mul2(p1, x3sp));                           // g1
-              pk[3][4 * hh + w] = pack_bf16x2(mul2(p3, a));                              // g3
-              pk[4][4 * hh + w] = pack_bf16x2(fma2(n1, t1, mul2(n3, d3a)));              // -dp
-              pk[5][4 * hh + w] = pack_bf16x2(mul2(n2, u));                              // -eta2 u
-              aq1 = fma2(pr, t1, aq1);
-              aq3 = fma2(pr, d3a, aq3);
-              aq2 = fma2(nd, u, aq2);
-            }
+            for (int q = 0; q < 6; ++q)
+#pragma unroll
+              for (int w = 0; w < 4; ++w) pk[q][4 * hh + w] = o[q][w];
           }
           if (valid) {
             const size_t off = (size_t)m * g.ld_out + f0 + c;
@@ -651,34 +1100,36 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
           }
         }
         if (valid)
-          store_deta(g, m, tn, -(x2_lo(aq1) + x2_hi(aq1)), -(x2_lo(aq3) + x2_hi(aq3)), -(x2_lo(aq2) + x2_hi(aq2)));
+          store_deta(g, m, tn, -(x2_lo(aq[0]) + x2_hi(aq[0])), -(x2_lo(aq[1]) + x2_hi(aq[1])),
+                     -(x2_lo(aq[2]) + x2_hi(aq[2])));
       } else {
-        // gate epilogues: columns [0, 128) are z1, [128, 256) z3 of hidden
-        // units f0 .. f0 + 127
-        const int f0 = tn * (BN / 2);
+        // gate epilogues: columns [0, 128) are z1, [128, 256) z3 of the tile's
+        // 128 hidden units; this warp's 64 from f0
         float e1 = 0.f, e3 = 0.f, e2 = 0.f;
         if (g.epi == EPI_KEY && valid) row_rates(g, m, e1, e3, e2);
         if (!g.mse) {   // dot loss: e = -eta v
           e1 = -e1;
           e3 = -e3;
         }
-        // this row's 128 values of the epilogue input (KEY: P; BAPPLY:
+        // this row's 64 values of the epilogue input (KEY: P; BAPPLY:
         // W2^T d_o), loaded at once: one memory latency per tile
-        uint4 prow[16];
+        const int f0 = tn * (BN / 2) + gp * (BN / 4);
+        const uint32_t acch = accb + gp * (BN / 4);
+        uint4 prow[8];
         if (g.epi != EPI_APPLY && valid) {
           const uint4* pp = reinterpret_cast<const uint4*>(g.in0 + (size_t)m * g.ld_out + f0);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) prow[j] = ldg16(pp + j);
+          for (int j = 0; j < 8; ++j) prow[j] = ldg16(pp + j);
         }
         // on pairs of hidden units (packed float32 lanes); KEY scales the
         // factors by the rates, BAPPLY by 1
         const bool key = g.epi == EPI_KEY;
-        const f32x2 s1 = x2(key ? e1 : 1.f), s3 = x2(key ? e3 : 1.f), s2 = x2(key ? -e2 : 1.f), one = x2(1.f);
+        const f32x2 s1 = x2(key ? e1 : 1.f), s3 = x2(key ? e3 : 1.f), s2 = x2(key ? -e2 : 1.f);
 #pragma unroll
-        for (int c = 0; c < BN / 2; c += 16) {
+        for (int c = 0; c < BN / 4; c += 16) {
           float z1[16], z3[16];
-          tmem_ld16(accb + c, z1);
-          tmem_ld16(accb + 128 + c, z3);
+          tmem_ld16(acch + c, z1);
+          tmem_ld16(acch + 128 + c, z3);
           if (!valid) continue;
           const size_t off = (size_t)m * g.ld_out + f0 + c;
           if (g.epi == EPI_APPLY) {
@@ -690,21 +1141,17 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
             }
             st_global_v8(reinterpret_cast<__nv_bfloat16*>(g.out[0]) + off, hw);
           } else {
-            float r[16];
-            unpack16(prow[c / 8], prow[c / 8 + 1], r);
             uint32_t w0[8], w1[8], w2[8];
 #pragma unroll
-            for (int w = 0; w < 8; ++w) {
-              const f32x2 x1 = x2(z1[2 * w], z1[2 * w + 1]), x3 = x2(z3[2 * w], z3[2 * w + 1]);
-              const f32x2 rr = x2(r[2 * w], r[2 * w + 1]);
-              const f32x2 sg = sigmoid2(x1);
-              const f32x2 a = mul2(x1, sg);
-              const f32x2 sp = fma2(a, sub2(one, sg), sg);        // silu'(z1)
-              // KEY: r = W2^T v (dot) or W2^T e (squared error) -> g1, g3, u~ = -eta2 u;
-              // BAPPLY: r = W2^T d_o -> dzq1, dzq3, uq
-              w0[w] = pack_bf16x2(mul2(mul2(mul2(s1, rr), x3), sp));
-              w1[w] = pack_bf16x2(mul2(mul2(s3, rr), a));
-              w2[w] = pack_bf16x2(mul2(s2, mul2(a, x3)));
+            for (int j = 0; j < 2; ++j) {
+              uint32_t o[3][4];
+              gate8(z1 + 8 * j, z3 + 8 * j, prow[c / 8 + j], s1, s3, s2, o);
+#pragma unroll
+              for (int w = 0; w < 4; ++w) {
+                w0[4 * j + w] = o[0][w];
+                w1[4 * j + w] = o[1][w];
+                w2[4 * j + w] = o[2][w];
+              }
             }
             st_global_v8(reinterpret_cast<__nv_bfloat16*>(g.out[0]) + off, w0);
             st_global_v8(reinterpret_cast<__nv_bfloat16*>(g.out[1]) + off, w1);
@@ -715,8 +1162,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
       // the accumulator is drained: the MMA warp may reuse it
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[gp]);
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(lead_empty + 8 * (i & 1));
+        else mbar_arrive(&acc_empty[i & 1]);
+      }
     }
+    if (PAIR && (!XSET || g.staged) && lane == 0) bulk_wait_all();
     // bounded-wait test: every tile is stored and no copy or MMA is in flight;
     // the wait runs out, raises the abort flag and the status word reports it
     if (g.timeout_test) mbar_wait(&never_bar, 0, abort, 50000000ull);
@@ -725,7 +1176,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) wide_gemm_kernel(const __grid
   __syncthreads();
   tc_fence_after();
   if (abort_flag && threadIdx.x == 0) atomicExch(g.status, SCAL3R_ERR_TIMEOUT);
-  if (warp == 1) tmem_dealloc(tb, 512);
+  if (PAIR) {
+    // neither CTA leaves, or frees TMEM, before the other has finished with it
+    // (every wait above is bounded, so both arrive)
+    cluster_sync();
+    tc_fence_after();
+    if (warp == 1) tmem_dealloc_pair(tb, 512);
+  } else if (warp == 1) {
+    tmem_dealloc(tb, 512);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1084,6 +1543,95 @@ int num_sms() {
   return n;
 }
 
+// The output maps of a staged epilogue (see OutStage); false if this epilogue
+// has no staged form or an output cannot be mapped (its base or row stride is
+// not a multiple of 16 bytes), then the outputs are stored directly.
+bool stage_outputs(GemmArgs& a) {
+#ifdef SCAL3R_DEBUG_BOUNDS
+  return false;   // the checked stores are the direct ones
+#else
+  auto fn = encode_fn();
+  if (!fn) return false;
+  auto map = [&](int i, int64_t cols, int64_t ld, bool f32, int box_cols, int64_t planes,
+                 int64_t plane, CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_128B) {
+    const cuuint64_t elt = f32 ? 4 : 2;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)a.M, (cuuint64_t)planes};
+    cuuint64_t strides[2] = {(cuuint64_t)ld * elt, (cuuint64_t)plane * elt};
+    cuuint32_t box[3] = {(cuuint32_t)box_cols, 32, 1};
+    cuuint32_t es[3] = {1, 1, 1};
+    return fn(&a.o[i], f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, a.out[i], dims,
+              strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  const int64_t one = (int64_t)a.M * a.ld_out;   // the stride of a third dimension of one plane
+  switch (a.epi) {
+    case EPI_F32:
+    case EPI_F32_ADD:
+    case EPI_F32_ADDIN:
+      return a.ksplit > 1 ? map(0, a.N, a.ld_out, true, 32, a.ksplit, a.split_stride)
+                          : map(0, a.N, a.ld_out, true, 32, 1, one);
+    case EPI_BF16: return map(0, a.N, a.ld_out, false, 64, 1, one);
+    case EPI_GCM_GATE:
+      return map(0, a.N, a.ld_out, false, 64, 1, one) && map(1, a.N, a.ld_out, false, 64, 1, one);
+    case EPI_GCM_QKV:
+      for (int i = 0; i < 3; ++i)
+        if (!map(i, a.ld_out, a.ld_out, false, 64, 1, one)) return false;
+      return true;
+    case EPI_BKEY:
+      for (int i = 0; i < 6; ++i)
+        if (!map(i, a.N / 4, a.ld_out, false, 16, 1, one, CU_TENSOR_MAP_SWIZZLE_32B)) return false;
+      return true;
+    default: return false;
+  }
+#endif
+}
+
+// The weight maps of a gate product for gate_tile: the hidden units of every 32
+// reordered (a 5-D view of the matrix whose box walks them as p, t, j of
+// f = 8 t + 2 j + p).  False if this is no gate product of that form.
+bool gate_maps(GemmArgs& a) {
+  const bool gate = a.epi == EPI_KEY || a.epi == EPI_BAPPLY || a.epi == EPI_APPLY;
+  auto fn = encode_fn();
+  if (!gate || !fn || !a.bw[0] || a.nbn != 2) return false;
+  const cuuint64_t row = (cuuint64_t)a.K * 2;
+  for (int i = 0; i < a.nbn; ++i) {
+    cuuint64_t dims[5] = {(cuuint64_t)a.K, 2, 4, 4, (cuuint64_t)(a.b_rows / 32)};
+    cuuint64_t strides[4] = {row, 8 * row, 2 * row, 32 * row};
+    cuuint32_t box[5] = {64, 2, 4, 4, BN / 2 / 32};
+    cuuint32_t es[5] = {1, 1, 1, 1, 1};
+    if (fn(&a.b[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.bw[i]), dims, strides, box, es,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return false;
+  }
+  a.gated = 1;
+  return true;
+}
+
+// CTA pairs or single CTAs: the fewer rounds of tiles, a pair's round (256 x
+// 256 outputs on two SMs) counted 0.9 of a single's (128 x 256 on each).
+bool use_pairs(int M, int64_t units, int64_t pairs, int64_t sms) {
+  if (M <= BM || sms < 2) return false;   // one row block: the pair's other half would be empty
+  const int64_t r1 = (units + sms - 1) / sms, r2 = (pairs + sms / 2 - 1) / (sms / 2);
+  return 10 * r1 > 9 * r2;
+}
+
+cudaError_t launch_pairs(void (*kernel)(const GemmArgs), const GemmArgs& a, int grid, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(GEMM_THREADS);
+  cfg.dynamicSmemBytes = PAIR_SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 cudaError_t gemm(GemmArgs& a, cudaStream_t st) {
   if (a.M <= 0 || a.N % BN != 0 || a.K <= 0) return cudaErrorInvalidValue;
   if (a.nseg < 1) a.nseg = 1;
@@ -1096,13 +1644,19 @@ cudaError_t gemm(GemmArgs& a, cudaStream_t st) {
   } else if (a.nseg > 1 || a.epi != EPI_F32 || a.kb_split < 1 || (int64_t)(a.ksplit - 1) * a.kb_split >= nk) {
     return cudaErrorInvalidValue;   // every K range non-empty, plain float32 partial planes only
   }
-  const int64_t units = (int64_t)((a.M + BM - 1) / BM) * (a.N / BN) * a.ksplit;
+  const int64_t tn = (int64_t)(a.N / BN) * a.ksplit, sms = num_sms();
+  const int64_t units = (a.M + BM - 1) / BM * tn, pairs = (a.M + 2 * BM - 1) / (2 * BM) * tn;
   if (units > INT32_MAX) return cudaErrorInvalidValue;
-  const int grid = (int)std::min<int64_t>(units, num_sms());
-  if ((a.epi >= EPI_MSE_E && a.epi <= EPI_APPLY2) || a.epi == EPI_BKEY)
-    wide_gemm_kernel<true><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(a);
-  else
-    wide_gemm_kernel<false><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(a);
+  const bool xset = (a.epi >= EPI_MSE_E && a.epi <= EPI_APPLY2) || a.epi == EPI_BKEY;
+  a.gated = a.staged = 0;
+  if (use_pairs(a.M, units, pairs, sms) && (gate_maps(a) || (a.staged = stage_outputs(a)) || xset)) {
+    const int grid = 2 * (int)std::min<int64_t>(pairs, sms / 2);
+    return xset ? launch_pairs(wide_gemm_kernel<true, true>, a, grid, st)
+                : launch_pairs(wide_gemm_kernel<false, true>, a, grid, st);
+  }
+  const int grid = (int)std::min<int64_t>(units, sms);
+  if (xset) wide_gemm_kernel<true, false><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(a);
+  else wide_gemm_kernel<false, false><<<grid, GEMM_THREADS, GEMM_SMEM, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1306,7 +1860,7 @@ cudaError_t wide_gcm_qkv(const void* x, const void* wqkv, const float* bqkv, int
   if (T <= 0) return cudaSuccess;
   if (d <= 0 || d % BN != 0 || T > INT32_MAX) return cudaErrorInvalidValue;
   GemmArgs g{};
-  if (!make_map(&g.a[0], x, T, 1, d, d, 128) || !make_map(&g.b[0], wqkv, 3 * (int64_t)d, 1, d, d, 256))
+  if (!make_map(&g.a[0], x, T, 1, d, d, 128) || !make_map(&g.b[0], wqkv, 3 * (int64_t)d, 1, d, d, 128))
     return cudaErrorInvalidValue;
   g.M = (int)T;
   g.N = 3 * d;
@@ -1329,7 +1883,7 @@ cudaError_t wide_gcm_gate(const void* o, const void* wo, const void* x, const fl
   if (T <= 0) return cudaSuccess;
   if (d <= 0 || d % BN != 0 || T > INT32_MAX) return cudaErrorInvalidValue;
   GemmArgs g{};
-  if (!make_map(&g.a[0], o, T, 1, d, d, 128) || !make_map(&g.b[0], wo, d, 1, d, d, 256))
+  if (!make_map(&g.a[0], o, T, 1, d, d, 128) || !make_map(&g.b[0], wo, d, 1, d, d, 128))
     return cudaErrorInvalidValue;
   g.M = (int)T;
   g.N = d;
@@ -1373,7 +1927,7 @@ cudaError_t wide_gemm_bf16(const void* a, int64_t lda, int a_kmajor, const void*
   const bool am = !a_kmajor, bm = !b_kmajor;
   if (!(am ? make_map(&g.a[0], a, K, 1, M, lda, 64) : make_map(&g.a[0], a, M, 1, K, lda, 128)))
     return cudaErrorInvalidValue;
-  if (!(bm ? make_map(&g.b[0], b, K, 1, N, ldb, 64) : make_map(&g.b[0], b, N, 1, K, ldb, 256)))
+  if (!(bm ? make_map(&g.b[0], b, K, 1, N, ldb, 64) : make_map(&g.b[0], b, N, 1, K, ldb, 128)))
     return cudaErrorInvalidValue;
   g.M = (int)M;
   g.N = (int)N;
@@ -1405,11 +1959,18 @@ cudaError_t wide_gemm_bf16(const void* a, int64_t lda, int a_kmajor, const void*
 }
 
 cudaError_t prepare_wide() {
-  cudaError_t e =
-      cudaFuncSetAttribute(wide_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wide_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
-  return e;
+  const struct {
+    const void* f;
+    size_t smem;
+  } ks[] = {{(const void*)wide_gemm_kernel<false, false>, GEMM_SMEM},
+            {(const void*)wide_gemm_kernel<true, false>, GEMM_SMEM},
+            {(const void*)wide_gemm_kernel<false, true>, PAIR_SMEM},
+            {(const void*)wide_gemm_kernel<true, true>, PAIR_SMEM}};
+  for (const auto& k : ks) {
+    const cudaError_t e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 namespace {
@@ -1437,12 +1998,13 @@ cudaError_t key_grad_mse(const Ctx& cx, int h, int c, const __nv_bfloat16* wb, f
     WIDE_MAP(tok_map(&a.a[0], prm.k, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
              mat_map(&a.b[1], w3, F, D, 128));
     a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+    a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
     a.epi = EPI_APPLY; a.out[0] = ub; a.ld_out = F;
     WIDE_TRY(run_gemm(cx, a, 2 * mfd));
   }
   {   // e = U W2^T - V and eta2 e
     GemmArgs a{};
-    WIDE_MAP(mat_map(&a.a[0], ub, M, F, 128) && mat_map(&a.b[0], w2, D, F, 256));
+    WIDE_MAP(mat_map(&a.a[0], ub, M, F, 128) && mat_map(&a.b[0], w2, D, F, 128));
     a.M = M; a.N = D; a.K = F;
     a.epi = EPI_MSE_E; a.out[0] = eb; a.out[1] = e2b; a.ld_out = D;
     a.in0 = reinterpret_cast<const __nv_bfloat16*>(prm.v) + ((size_t)t0 * H + h) * D; a.ld_in = (int64_t)H * D;
@@ -1461,6 +2023,7 @@ cudaError_t key_grad_mse(const Ctx& cx, int h, int c, const __nv_bfloat16* wb, f
     WIDE_MAP(tok_map(&a.a[0], prm.k, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
              mat_map(&a.b[1], w3, F, D, 128));
     a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+    a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
     a.epi = EPI_KEY; a.mse = 1; a.out[0] = g1; a.out[1] = g3; a.ld_out = F; a.in0 = pb;
     set_rates(a, prm, t0, h);
     WIDE_TRY(run_gemm(cx, a, 2 * mfd));
@@ -1511,6 +2074,7 @@ cudaError_t key_grad(const Ctx& cx, int h, int c, const __nv_bfloat16* wb, float
     WIDE_MAP(tok_map(&a.a[0], prm.k, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
              mat_map(&a.b[1], w3, F, D, 128));
     a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+    a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
     a.epi = EPI_KEY; a.out[0] = g1; a.out[1] = g3; a.out[2] = ut; a.ld_out = F; a.in0 = pb;
     set_rates(a, prm, t0, h);
     WIDE_TRY(run_gemm(cx, a, 2 * mfd));
@@ -1590,12 +2154,13 @@ cudaError_t wide_forward(const Plan& pl, const Shape& sh, const Params& prm, int
           WIDE_MAP(tok_map(&a.a[0], prm.q, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
                    mat_map(&a.b[1], w3, F, D, 128));
           a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+          a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
           a.epi = EPI_APPLY; a.out[0] = pb; a.ld_out = F;
           WIDE_TRY(run_gemm(cx, a, 2 * mfd));
         }
         {   // o = h W2^T
           GemmArgs a{};
-          WIDE_MAP(mat_map(&a.a[0], pb, M, F, 128) && mat_map(&a.b[0], w2, D, F, 256));
+          WIDE_MAP(mat_map(&a.a[0], pb, M, F, 128) && mat_map(&a.b[0], w2, D, F, 128));
           a.M = M; a.N = D; a.K = F;
           a.epi = EPI_BF16; a.out[0] = reinterpret_cast<__nv_bfloat16*>(prm.o) + ((size_t)t0 * H + h) * D;
           a.ld_out = (int64_t)H * D;
@@ -1721,12 +2286,13 @@ cudaError_t wide_apply(const Plan& pl, const Shape& sh, const Params& prm, void*
         WIDE_MAP(tok_map(&a.a[0], prm.q, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
                  mat_map(&a.b[1], w3, F, D, 128));
         a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+        a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
         a.epi = EPI_APPLY; a.out[0] = pb; a.ld_out = F;
         WIDE_TRY(run_gemm(cx, a, 2 * mfd));
       }
       {
         GemmArgs a{};
-        WIDE_MAP(mat_map(&a.a[0], pb, M, F, 128) && mat_map(&a.b[0], w2, D, F, 256));
+        WIDE_MAP(mat_map(&a.a[0], pb, M, F, 128) && mat_map(&a.b[0], w2, D, F, 128));
         a.M = M; a.N = D; a.K = F;
         a.epi = EPI_BF16; a.out[0] = reinterpret_cast<__nv_bfloat16*>(prm.o) + ((size_t)t0 * H + h) * D;
         a.ld_out = (int64_t)H * D;
@@ -1773,7 +2339,7 @@ cudaError_t update_vjp_mse(const Ctx& cx, int h, int64_t t0, int M, const WideBu
   }
   {   // e = U W2^T - V
     GemmArgs a{};
-    WIDE_MAP(mat_map(&a.a[0], ub, M, F, 128) && mat_map(&a.b[0], w2, D, F, 256));
+    WIDE_MAP(mat_map(&a.a[0], ub, M, F, 128) && mat_map(&a.b[0], w2, D, F, 128));
     a.M = M; a.N = D; a.K = F;
     a.epi = EPI_MSE_E; a.out[0] = eb; a.ld_out = D;
     a.in0 = reinterpret_cast<const __nv_bfloat16*>(prm.v) + ((size_t)t0 * H + h) * D; a.ld_in = (int64_t)H * D;
@@ -1791,7 +2357,7 @@ cudaError_t update_vjp_mse(const Ctx& cx, int h, int64_t t0, int M, const WideBu
       {   // dE = -eta2 U R2^T + dP W2^T -> dY, dv
         GemmArgs a{};
         WIDE_MAP(mat_map(&a.a[0], u2, M, F, 128) && mat_map(&a.a[1], dp, M, F, 128) &&
-                 mat_map(&a.b[0], r2, D, F, 256) && mat_map(&a.b[1], w2, D, F, 256));
+                 mat_map(&a.b[0], r2, D, F, 128) && mat_map(&a.b[1], w2, D, F, 128));
         a.M = M; a.N = D; a.K = 2 * F; a.kseg = F; a.nseg = 2;
         a.epi = EPI_MSE_DE; a.out[0] = dy; a.ld_out = D;
         a.out[1] = reinterpret_cast<__nv_bfloat16*>(prm.dv) + ((size_t)t0 * H + h) * D; a.ld_out1 = (int64_t)H * D;
@@ -1932,6 +2498,7 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
             WIDE_MAP(tok_map(&a.a[0], prm.q, T, H, D, 128) && mat_map(&a.b[0], w1, F, D, 128) &&
                      mat_map(&a.b[1], w3, F, D, 128));
             a.M = M; a.N = 2 * F; a.K = D; a.nbn = 2; a.ha = h; a.ya = (int)t0;
+            a.bw[0] = w1; a.bw[1] = w3; a.b_rows = F;
             a.epi = EPI_BAPPLY; a.out[0] = dz1; a.out[1] = dz3; a.out[2] = uq; a.ld_out = F; a.in0 = du;
             WIDE_TRY(run_gemm(cx, a, 2 * mfd));
           }
@@ -2007,7 +2574,7 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
           {   // dv = [-dp, -eta2 u] [W2^T; -R2^T]
             GemmArgs a{};
             WIDE_MAP(mat_map(&a.a[0], dpe, M, F, 128) && mat_map(&a.a[1], ue, M, F, 128) &&
-                     mat_map(&a.b[0], w2, D, F, 256) && mat_map(&a.b[1], r2, D, F, 256));
+                     mat_map(&a.b[0], w2, D, F, 128) && mat_map(&a.b[1], r2, D, F, 128));
             a.M = M; a.N = D; a.K = 2 * F; a.kseg = F; a.nseg = 2;
             a.epi = EPI_BF16; a.out[0] = reinterpret_cast<__nv_bfloat16*>(prm.dv) + ((size_t)t0 * H + h) * D;
             a.ld_out = (int64_t)H * D;
