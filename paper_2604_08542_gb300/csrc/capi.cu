@@ -173,7 +173,8 @@ void free_plan(Plan& p) {
   if (p.d_bupdates) cudaFree(p.d_bupdates);
   if (p.d_ritems) cudaFree(p.d_ritems);
   if (p.d_yitems) cudaFree(p.d_yitems);
-  p.d_yitems = nullptr;
+  if (p.d_bresid) cudaFree(p.d_bresid);
+  p.d_yitems = p.d_bresid = nullptr;
   if (p.d_rupdates) cudaFree(p.d_rupdates);
   if (p.d_segsrc) cudaFree(p.d_segsrc);
   p.d_ritems = nullptr;
@@ -239,7 +240,8 @@ int ensure_plan(scal3r_ttt_handle* hd, const int64_t* off, int32_t C, const int3
       upload(&np.d_bitems, np.bitems) != cudaSuccess || upload(&np.d_bupdates, np.bupdates) != cudaSuccess ||
       upload(&np.d_off, np.chunk_offsets) != cudaSuccess || upload(&np.d_ptr, np.seq_chunk_ptr) != cudaSuccess ||
       upload(&np.d_ritems, np.ritems) != cudaSuccess || upload(&np.d_rupdates, np.rupdates) != cudaSuccess ||
-      upload(&np.d_segsrc, np.segsrc) != cudaSuccess || upload(&np.d_yitems, np.yitems) != cudaSuccess) {
+      upload(&np.d_segsrc, np.segsrc) != cudaSuccess || upload(&np.d_yitems, np.yitems) != cudaSuccess ||
+      upload(&np.d_bresid, np.bresid) != cudaSuccess) {
     free_plan(np);
     return SCAL3R_ERR_CUDA;
   }
@@ -468,7 +470,8 @@ int enqueue_backward(scal3r_ttt_handle* hd, const Params& prm, cudaStream_t st) 
     const WorkItem* post = pl.d_bitems + s.item0 + nmain;
     Params pm = pb;
     if (s.npost > 0) {
-      if (run_resid(hd, pb, pl.bitems.data() + s.item0 + nmain, post, s.npost, (int)j, true, st) != cudaSuccess)
+      if (run_resid(hd, pb, pl.bresid.data() + s.bres0, pl.d_bresid + s.bres0, s.nbres, (int)j, true, st) !=
+          cudaSuccess)
         return SCAL3R_ERR_CUDA;
       pm.v = prm.rtok;
     }

@@ -429,6 +429,18 @@ int build_plan(Plan& plan, const Shape& s, const Schedule& sch_in, int num_sms,
       auto mid = std::stable_partition(first, first + bs.nitems,
                                        [](const WorkItem& w) { return w.role != ROLE_BAPPLY_K; });
       bs.npost = (int32_t)(first + bs.nitems - mid);
+      bs.bres0 = (int32_t)p.bresid.size();
+      const int per = bs.npost > 0 ? std::max(1, num_sms / bs.npost) : 1;
+      for (auto it = mid; it != first + bs.nitems; ++it)
+        for (auto& pr : split(it->t0, it->t1, per, sch.align)) {
+          WorkItem y = *it;
+          y.t0 = pr.first;
+          y.t1 = pr.second;
+          y.role = ROLE_APPLY;
+          y.slot = -1;
+          p.bresid.push_back(y);
+        }
+      bs.nbres = (int32_t)p.bresid.size() - bs.bres0;
     }
     if (nck > 1 && j % nck != 0) {
       bs.wseg = j % nck;

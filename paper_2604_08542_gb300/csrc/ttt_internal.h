@@ -61,6 +61,7 @@ struct Step {
   int32_t segk = 0;       //   whose sources are row segk of the plan's segment table
   int32_t npost = 0;      // backward, composed squared-error loss: the last npost pieces are
                           // ROLE_BAPPLY_K, launched after the others
+  int32_t bres0 = 0, nbres = 0;   // backward, composed squared-error loss: the residual pieces of those chunks
   int32_t nfill = 0;      // tail fill: the last nfill pieces (before any npost) start behind
                           // the first wave, in the order their SMs are modelled to free
 };
@@ -95,6 +96,8 @@ struct Plan {
   // token ranges, as apply pieces)
   bool mse_compose = false;
   std::vector<WorkItem> yitems;
+  std::vector<WorkItem> bresid;     // per backward step, the same over the SMs (an apply piece's rows are
+                                    // independent, so its cut is free; the key-side VJPs' is the sums' order)
   std::vector<Step> ysteps;
   // device copies (owned by the handle)
   WorkItem* d_items = nullptr;
@@ -103,6 +106,7 @@ struct Plan {
   UpdateItem* d_bupdates = nullptr;
   WorkItem* d_ritems = nullptr;
   WorkItem* d_yitems = nullptr;
+  WorkItem* d_bresid = nullptr;
   UpdateItem* d_rupdates = nullptr;
   int32_t* d_segsrc = nullptr;
   int64_t* d_off = nullptr;     // chunk_offsets and seq_chunk_ptr (the linear model's kernels)
