@@ -2,8 +2,7 @@
 // schedule cache and the launch sequence of one forward / backward call.
 //
 // Forward, for a layout whose longest sequence has n chunks:
-//   prep (copy w0, row-norm targets)
-//   for j = 0 .. n:  sweep(j)   gradient pieces of chunk j + apply pieces of
+//   for j = 0 .. n (at j = 0 from w0 itself):  sweep(j)   gradient pieces of chunk j + apply pieces of
 //                               chunk j-1, all at the weights W_j
 //                    update(j)  W_{j+1} = normalise(W_j + sum of pieces)
 // Backward, for j = n .. 0: sweep(j) (VJP pieces of chunk j's update and
@@ -378,9 +377,6 @@ cudaError_t run_resid(scal3r_ttt_handle* hd, const Params& prm, const WorkItem* 
 
 int enqueue_forward(scal3r_ttt_handle* hd, const Params& prm, cudaStream_t st) {
   const Plan& pl = hd->plan;
-  const int chains = pl.S * hd->shape.H;
-  if (timed(hd, SCAL3R_KERNEL_OTHER, 0, 0, st, [&] { return launch_prep(prm, chains, st); }) != cudaSuccess)
-    return SCAL3R_ERR_CUDA;
   Params pk = prm;   // the gradient pieces see the residuals as their values
   if (pl.mse_compose) {
     pk.v = prm.rtok;
@@ -391,9 +387,11 @@ int enqueue_forward(scal3r_ttt_handle* hd, const Params& prm, cudaStream_t st) {
   }
   for (size_t j = 0; j < pl.steps.size(); ++j) {
     const Step& s = pl.steps[j];
+    Params pu = prm;
+    pk.w_items = pu.w_items = j == 0;   // the first step runs on w0 itself
     if (pl.mse_compose) {
       const Step& ys = pl.ysteps[j];
-      if (run_resid(hd, prm, pl.yitems.data() + ys.item0, pl.d_yitems + ys.item0, ys.nitems, (int)j, false, st) !=
+      if (run_resid(hd, prm, pl.yitems.data() + ys.item0, pl.d_yitems + ys.item0, ys.nitems, (int)j, j == 0, st) !=
           cudaSuccess)
         return SCAL3R_ERR_CUDA;
     }
@@ -407,7 +405,7 @@ int enqueue_forward(scal3r_ttt_handle* hd, const Params& prm, cudaStream_t st) {
       });
     if (e != cudaSuccess) return SCAL3R_ERR_CUDA;
     if (s.nupd > 0 && timed(hd, SCAL3R_KERNEL_FWD_UPDATE, 0, 0, st, [&] {
-          return launch_update(prm, pl.d_updates + s.upd0, s.nupd, (int)j, st);
+          return launch_update(pu, pl.d_updates + s.upd0, s.nupd, (int)j, st);
         }) != cudaSuccess)
       return SCAL3R_ERR_CUDA;
   }
@@ -1210,15 +1208,13 @@ int scal3r_ttt_partial_grad(scal3r_ttt_handle* hd, const void* k, const void* v,
   prm.w0_seq_stride = w_seq_stride;
   carve_workspace(pl, sh, false, workspace, prm);
   cudaStream_t st = (cudaStream_t)stream;
-  const int chains = pl.S * sh.H;
-  if (timed(hd, SCAL3R_KERNEL_OTHER, 0, 0, st, [&] { return launch_prep(prm, chains, st); }) != cudaSuccess)
-    return SCAL3R_ERR_CUDA;
+  prm.w_items = 1;   // the pieces read w itself
   const Step& s0 = pl.steps[0];   // the gradient pieces of every sequence's chunk, at w
   Params pk = prm;
   if (pl.mse_compose) {   // residuals first; the gradient pieces see them as values
     if (cudaMemsetAsync(prm.rtok, 0, (size_t)pl.T * sh.H * sh.D * 2, st) != cudaSuccess) return SCAL3R_ERR_CUDA;
     const Step& ys = pl.ysteps[0];
-    if (run_resid(hd, prm, pl.yitems.data() + ys.item0, pl.d_yitems + ys.item0, ys.nitems, 0, false, st) !=
+    if (run_resid(hd, prm, pl.yitems.data() + ys.item0, pl.d_yitems + ys.item0, ys.nitems, 0, true, st) !=
         cudaSuccess)
       return SCAL3R_ERR_CUDA;
     pk.v = prm.rtok;
@@ -1314,10 +1310,7 @@ int scal3r_ttt_apply(scal3r_ttt_handle* hd, const void* q, const float* w, int64
   prm.w0_seq_stride = w_seq_stride;
   carve_workspace(pl, sh, false, workspace, prm);
   cudaStream_t st = (cudaStream_t)stream;
-  const int chains = pl.S * sh.H;
-  // chunk step 1 applies each sequence's chunk with master buffer 1
-  if (timed(hd, SCAL3R_KERNEL_OTHER, 0, 0, st, [&] { return launch_loadw(prm, chains, 1, st); }) != cudaSuccess)
-    return SCAL3R_ERR_CUDA;
+  prm.w_items = 1;   // the pieces read w itself; chunk step 1 applies each sequence's chunk
   const Step& s1 = pl.steps[1];
   double fl = 0, by = 0;
   if (hd->prof_on) sweep_work(hd, pl.items.data() + s1.item0, s1.nitems, fl, by);

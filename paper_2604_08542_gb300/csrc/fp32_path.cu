@@ -115,7 +115,8 @@ fp32_sweep_kernel(Params p, const WorkItem* __restrict__ items, int step) {
   const int h = it.chain % H;
   const int chains = p.S * H;
   const int nr = p.lr_mat ? 3 : 1;
-  const float* w = p.wm + ((size_t)(step & 1) * chains + it.chain) * 3 * F * D;
+  const float* w = p.w_items ? p.w0 + (size_t)(it.chain / H) * p.w0_seq_stride + (size_t)h * 3 * F * D
+                             : p.wm + ((size_t)(step & 1) * chains + it.chain) * 3 * F * D;
   load_weights<D, F>(sm, w);
   const int tid = threadIdx.x;
 

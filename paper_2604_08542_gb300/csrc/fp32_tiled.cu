@@ -492,7 +492,8 @@ __global__ void __launch_bounds__(NTH, 1) fp32_tiled_sweep(Params p, const WorkI
   extern __shared__ __align__(16) float smf[];
   pdl_wait();   // the step's weights come from the kernel ahead of this one
   const WorkItem it = items[blockIdx.x];
-  const float* w = p.wm + ((size_t)(step & 1) * p.S * p.H + it.chain) * P;
+  const float* w = p.w_items ? p.w0 + (size_t)(it.chain / p.H) * p.w0_seq_stride + (size_t)(it.chain % p.H) * P
+                             : p.wm + ((size_t)(step & 1) * p.S * p.H + it.chain) * P;
   if (it.role == ROLE_APPLY) run_apply(p, it, w, smf);
   else run_token_pass<false>(p, it, w, smf);
 }

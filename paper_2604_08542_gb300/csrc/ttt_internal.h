@@ -190,7 +190,8 @@ struct Params {
   void* rtok;       // composed squared-error loss: [T][H][D] bf16 residuals r = v - f_W(k), then -dr
   void* dk2;        //   backward: [T][H][D] bf16 dk of the apply VJP over the keys
   const void* resid_v;   // apply pieces write v - f_W(x) instead of f_W(x) (values v)
-  int32_t w_items;  // 1: forward pieces read their weights as the backward does (wchunk)
+  int32_t w_items;  // 1: forward pieces read their weights as the backward does (wchunk; -1: w0), and
+                    //    the update of such a step starts from w0
   void* scratch;    // backward, BF16 path: per-piece factors of the weight adjoints
   int64_t scratch_tiles;   // its size in 96 KB tiles
   int* status;      // handle-owned status word
@@ -215,7 +216,6 @@ cudaError_t launch_update(const Params& prm, const UpdateItem* upd, int nupd, in
 cudaError_t launch_bupdate(const Params& prm, const UpdateItem* upd, int nupd, int step, cudaStream_t st);
 cudaError_t launch_bfinal(const Params& prm, cudaStream_t st);
 cudaError_t launch_gsum(const Params& prm, const UpdateItem* upd, int nupd, float* grad, cudaStream_t st);
-cudaError_t launch_loadw(const Params& prm, int chains, int buf, cudaStream_t st);
 cudaError_t launch_tok_negate(const Params& prm, const WorkItem* items, int nitems, const void* src, void* dst,
                               cudaStream_t st);
 cudaError_t launch_tok_add(const Params& prm, const WorkItem* items, int nitems, void* acc, const void* add,

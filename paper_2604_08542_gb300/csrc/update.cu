@@ -69,6 +69,13 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 __device__ __forceinline__ float4 scale4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
 __device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
+// The sum of squares of four elements with its rounding written out: a row's
+// target is formed from w0 by several kernels, which have to agree to the bit
+// (the backward's recomputed weights are the forward's).
+__device__ __forceinline__ float sumsq4(float4 a) {
+  return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.x, a.x, __fmul_rn(a.y, a.y))));
+}
+
 // x + the slots slot0 .. slot0 + n - 1 at element offset `off`, added one by
 // one in slot order (fixed-order reduction); the loads of a batch of eight
 // slots are issued before any of them is added, so the sum costs one memory
@@ -97,7 +104,7 @@ __device__ __forceinline__ float row_target(const Params& p, float ss) {
 }
 
 // Copy the starting weights of every chain into master buffer 0 and compute
-// the row-norm targets.
+// the row-norm targets (the allocation-free forward only, see update_kernel).
 __global__ void prep_kernel(Params p) {
   pdl_wait();
   const int chain = blockIdx.x;
@@ -106,13 +113,16 @@ __global__ void prep_kernel(Params p) {
   const float* w0 = chain_w0(p, chain);
   float4 w = s.valid ? ld4(w0 + s.off) : make_float4(0.f, 0.f, 0.f, 0.f);
   if (s.valid) st4(p.wm + (size_t)chain * P + s.off, w);
-  const float ss = group_sum(dot4(w, w), s.group);
+  const float ss = group_sum(sumsq4(w), s.group);
   if (s.valid && s.c4 == 0) st_chk(p.rho + (size_t)chain * R + s.r, row_target(p, ss));
 }
 
 // Forward update of one chain at step `step`:
 //   W~ = W_step + sum_slots partial (fixed slot order),
 //   W_{step+1} row = W~ row * rho / max(||W~ row||, eps).
+// With w_items (a forward's first step) W_step is w0 itself and the row targets
+// come from it here, so that no launch copies w0 first (3.6 us and its launch on
+// every forward call).
 __global__ void update_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
   pdl_wait();
   const UpdateItem u = upd[blockIdx.x];
@@ -120,19 +130,24 @@ __global__ void update_kernel(Params p, const UpdateItem* __restrict__ upd, int 
   const int P = 3 * p.F * p.D, R = 2 * p.F + p.D;
   const int chains = p.S * p.H;
   const int h = u.chain % p.H;
-  const float* wcur = p.wm + ((size_t)(step & 1) * chains + u.chain) * P;
+  const float* wcur = p.w_items ? chain_w0(p, u.chain) : p.wm + ((size_t)(step & 1) * chains + u.chain) * P;
   float* wnext = p.wm + ((size_t)((step + 1) & 1) * chains + u.chain) * P;
   if (u.chunk < 0) {   // sequence without chunks: w_final = w0
     if (p.w_final && s.valid) st4(p.w_final + ((size_t)u.seq * p.H + h) * P + s.off, ld4(wcur + s.off));
     return;
   }
-  float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 x = make_float4(0.f, 0.f, 0.f, 0.f), w0 = x;
   float rho = 1.f;
   if (s.valid) {
     // the row target is loaded before the slot sum so that its round trip
     // overlaps the sum's
-    if (p.norm != SCAL3R_NORM_NONE) rho = ld_chk(p.rho + (size_t)u.chain * R + s.r);
-    x = add_slots(ld4(wcur + s.off), p.part, u.slot0, u.nslots, P, s.off);
+    if (p.norm != SCAL3R_NORM_NONE && !p.w_items) rho = ld_chk(p.rho + (size_t)u.chain * R + s.r);
+    w0 = ld4(wcur + s.off);
+    x = add_slots(w0, p.part, u.slot0, u.nslots, P, s.off);
+  }
+  if (p.w_items && p.norm != SCAL3R_NORM_NONE) {   // the chain's first update: the row targets, kept for the next ones
+    rho = row_target(p, group_sum(sumsq4(w0), s.group));
+    if (s.valid && s.c4 == 0) st_chk(p.rho + (size_t)u.chain * R + s.r, rho);
   }
   const float n = sqrtf(group_sum(dot4(x, x), s.group));
   if (!s.valid) return;
@@ -155,7 +170,7 @@ __global__ void bprep_kernel(Params p) {
   const float* w0 = chain_w0(p, chain);
   const float4 w = s.valid ? ld4(w0 + s.off) : make_float4(0.f, 0.f, 0.f, 0.f);
   if (s.valid) st4(p.dw0_chain + (size_t)chain * P + s.off, make_float4(0.f, 0.f, 0.f, 0.f));
-  const float ss = group_sum(dot4(w, w), s.group);
+  const float ss = group_sum(sumsq4(w), s.group);
   if (s.valid && s.c4 == 0) {
     st_chk(p.rho + (size_t)chain * R + s.r, row_target(p, ss));
     st_chk(p.drho + (size_t)chain * R + s.r, 0.f);
@@ -260,15 +275,6 @@ __global__ void gsum_kernel(Params p, const UpdateItem* __restrict__ upd, float*
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
   if (u.chunk >= 0) x = add_slots(x, p.part, u.slot0, u.nslots, P, s.off);
   st4(grad + ((size_t)u.seq * p.H + h) * P + s.off, scale4(x, -1.f));
-}
-
-// The weights given in (w0, w0_seq_stride) into master buffer `buf`.
-__global__ void loadw_kernel(Params p, int buf) {
-  const int chain = blockIdx.x;
-  const RowSlice s = row_slice(blockIdx.y, p.D, p.F);
-  if (!s.valid) return;
-  const int P = 3 * p.F * p.D;
-  st4(p.wm + ((size_t)buf * p.S * p.H + chain) * P + s.off, ld4(chain_w0(p, chain) + s.off));
 }
 
 // Token rows of the pieces' ranges (head of the piece's chain) of a bf16
@@ -384,12 +390,6 @@ cudaError_t launch_bprep(const Params& prm, int chains, cudaStream_t st) {
 cudaError_t launch_gsum(const Params& prm, const UpdateItem* upd, int nupd, float* grad, cudaStream_t st) {
   if (nupd == 0) return cudaSuccess;
   gsum_kernel<<<dim3(nupd, row_blocks(prm)), kThreads, 0, st>>>(prm, upd, grad);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_loadw(const Params& prm, int chains, int buf, cudaStream_t st) {
-  if (chains == 0) return cudaSuccess;
-  loadw_kernel<<<dim3(chains, row_blocks(prm)), kThreads, 0, st>>>(prm, buf);
   return cudaGetLastError();
 }
 
