@@ -51,6 +51,12 @@ __device__ __forceinline__ void unpack8(const uint4 w, float (&f)[8]) {
     f[2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u);
   }
 }
+__device__ __forceinline__ void unpack4(const uint2 w, float (&f)[4]) {
+  f[0] = __uint_as_float(w.x << 16);
+  f[1] = __uint_as_float(w.x & 0xFFFF0000u);
+  f[2] = __uint_as_float(w.y << 16);
+  f[3] = __uint_as_float(w.y & 0xFFFF0000u);
+}
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
@@ -156,10 +162,10 @@ __global__ void __launch_bounds__(256) gcm_norm_eta_kernel(const float* __restri
 // unit-norm q the layer saw), [2d, 3d) dv, then dlogit = dlr base s (1 - s)
 // for heads h < H and zeros to column 3d + 63.  A head's D values are G =
 // min(32, D/8) lanes' chunks; G lanes reduce its dot with xor shuffles inside
-// their aligned group, 32/G heads at a time.  Block b takes the kRowBlock
-// tokens from b * kRowBlock; once its rows are written (and still in L2) it
-// sums them per column, in token order, into part[b][ld] (the partial rows of
-// dbqkv and db_eta).
+// their aligned group, 32/G heads at a time.  Bound by memory (about 16 d bytes
+// a token); the column sums of ext are colsum_part_kernel's.  (One block per 128
+// tokens that also summed its rows' columns left 131 blocks of 8 warps for 16,656
+// tokens: 150 us at d = 1024, against 49 + 21 us for the two kernels.)
 __global__ void __launch_bounds__(256) gcm_qkv_bwd_kernel(const __nv_bfloat16* __restrict__ dq,
                                                           const __nv_bfloat16* __restrict__ dk,
                                                           const __nv_bfloat16* __restrict__ dv,
@@ -168,13 +174,12 @@ __global__ void __launch_bounds__(256) gcm_qkv_bwd_kernel(const __nv_bfloat16* _
                                                           const __nv_bfloat16* __restrict__ k,
                                                           const float* __restrict__ qn, const float* __restrict__ kn,
                                                           const float* __restrict__ sig, float base, int64_t T, int H,
-                                                          int D, __nv_bfloat16* __restrict__ ext,
-                                                          float* __restrict__ part) {
+                                                          int D, __nv_bfloat16* __restrict__ ext) {
   const int lane = threadIdx.x & 31, d = H * D, nc = d / 8, cph = D / 8;
   const int G = cph < 32 ? cph : 32, hpi = 32 / G, per = cph / G;
   const size_t ld = 3 * (size_t)d + kEtaPad;
-  const int64_t t0 = (int64_t)blockIdx.x * kRowBlock, t1 = min(T, t0 + kRowBlock);
-  for (int64_t t = t0 + threadIdx.x / 32; t < t1; t += blockDim.x / 32) {
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x / 32);
+  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; t < T; t += step) {
     __nv_bfloat16* out = ext + (size_t)t * ld;
     for (int part = 0; part < 2; ++part) {
       const uint4* gg = reinterpret_cast<const uint4*>((part ? dk : dq) + (size_t)t * d);
@@ -216,51 +221,36 @@ __global__ void __launch_bounds__(256) gcm_qkv_bwd_kernel(const __nv_bfloat16* _
       out[3 * (size_t)d + col] = __float2bfloat16(g);
     }
   }
-  // the block's rows are written: their column sums, 8 columns per thread
-  __syncthreads();
-  for (int v = threadIdx.x; v < (int)(ld / 8); v += blockDim.x) {
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    for (int64_t t = t0; t < t1; ++t) {
-      float f[8];
-      unpack8(reinterpret_cast<const uint4*>(ext + (size_t)t * ld)[v], f);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] += f[e];
-    }
-    float4* o = reinterpret_cast<float4*>(part + (size_t)blockIdx.x * ld + 8 * v);
-    o[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-    o[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
-  }
 }
 
 // Per kRowBlock-token block, column sums of a bf16 [T][ncol] array (or of the
-// product of two) into part[block][ncol]; one thread per 8 columns.
+// product of two) into part[block][ncol]; one thread per 4 columns, 16 tokens'
+// loads in flight, added in token order.  Bound by those loads' latency: few
+// threads carry a sum (8 columns a thread: 32 us for 16,656 x 3,136 columns and
+// 41 us for the product of two 16,656 x 1,024; here 21 and 34).
 template <bool PROD>
-__global__ void colsum8_part_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __restrict__ b,
-                                    int64_t T, int ncol, float* __restrict__ part) {
+__global__ void __launch_bounds__(64) colsum_part_kernel(const __nv_bfloat16* __restrict__ a,
+                                                         const __nv_bfloat16* __restrict__ b, int64_t T, int ncol,
+                                                         float* __restrict__ part) {
   const int v = blockIdx.y * blockDim.x + threadIdx.x;
-  if (8 * v >= ncol) return;
+  if (4 * v >= ncol) return;
   const int64_t t0 = (int64_t)blockIdx.x * kRowBlock, t1 = min(T, t0 + kRowBlock);
-  float s[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) s[e] = 0.f;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
   for (int64_t t = t0; t < t1; ++t) {
-    float f[8];
-    unpack8(reinterpret_cast<const uint4*>(a + (size_t)t * ncol)[v], f);
+    float f[4];
+    unpack4(reinterpret_cast<const uint2*>(a + (size_t)t * ncol)[v], f);
     if (PROD) {
-      float g[8];
-      unpack8(reinterpret_cast<const uint4*>(b + (size_t)t * ncol)[v], g);
+      float g[4];
+      unpack4(reinterpret_cast<const uint2*>(b + (size_t)t * ncol)[v], g);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) s[e] = fmaf(f[e], g[e], s[e]);
+      for (int e = 0; e < 4; ++e) s[e] = fmaf(f[e], g[e], s[e]);
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) s[e] += f[e];
+      for (int e = 0; e < 4; ++e) s[e] += f[e];
     }
   }
-  float4* o = reinterpret_cast<float4*>(part + (size_t)blockIdx.x * ncol + 8 * v);
-  o[0] = make_float4(s[0], s[1], s[2], s[3]);
-  o[1] = make_float4(s[4], s[5], s[6], s[7]);
+  *reinterpret_cast<float4*>(part + (size_t)blockIdx.x * ncol + 4 * v) = make_float4(s[0], s[1], s[2], s[3]);
 }
 
 // Column sums of `rows` partial rows (`stride` floats apart), columns
@@ -387,7 +377,7 @@ cudaError_t gcm_out_backward(const void* d_out, const void* o, const void* wo, c
   if (e == cudaSuccess) e = wide_gemm_bf16(d_out, d, 0, o, d, 0, dwo, d, 1, 0, d, d, T, c, gwb, 0, status, st);
   if (e != cudaSuccess) return e;
   scale_rows_f32_kernel<<<grid_of((int64_t)d * d, 256, 4 * sms), 256, 0, st>>>(dwo, alpha, d, d);
-  colsum8_part_kernel<true><<<dim3((unsigned)nb, (d / 8 + 255) / 256), 256, 0, st>>>(
+  colsum_part_kernel<true><<<dim3((unsigned)nb, (d / 4 + 63) / 64), 64, 0, st>>>(
       static_cast<const __nv_bfloat16*>(y), static_cast<const __nv_bfloat16*>(d_out), T, d, part);
   colsum_kernel<<<(d + 31) / 32, 32 * kColsumWarps, 0, st>>>(part, nb, d, d, dalpha);
   return cudaGetLastError();
@@ -425,9 +415,10 @@ cudaError_t gcm_qkv_backward(const void* dq, const void* dk, const void* dv, con
   void* gws2 = c;   // the split planes of the dw_eta product (its own region: it splits, dWqkv may not)
   const size_t gwb2 = wide_gemm_workspace_bytes(kEtaPad, d, T, 1);
   using bf = __nv_bfloat16;
-  gcm_qkv_bwd_kernel<<<(unsigned)nb, 256, 0, st>>>(
+  gcm_qkv_bwd_kernel<<<grid_of(T, 8, 8 * sms), 256, 0, st>>>(
       static_cast<const bf*>(dq), static_cast<const bf*>(dk), static_cast<const bf*>(dv), dlr,
-      static_cast<const bf*>(q), static_cast<const bf*>(k), qn, kn, sig, base, T, H, D, ext, part);
+      static_cast<const bf*>(q), static_cast<const bf*>(k), qn, kn, sig, base, T, H, D, ext);
+  colsum_part_kernel<false><<<dim3((unsigned)nb, (ld / 4 + 63) / 64), 64, 0, st>>>(ext, nullptr, T, ld, part);
   colsum_kernel<<<(3 * d + 31) / 32, 32 * kColsumWarps, 0, st>>>(part, nb, ld, 3 * d, dbqkv);
   colsum_kernel<<<1, 32 * kColsumWarps, 0, st>>>(part + 3 * d, nb, ld, H, db_eta);
   cudaError_t e = cudaMemcpyAsync(bext, wqkv, (size_t)3 * d * d * 2, cudaMemcpyDeviceToDevice, st);

@@ -1252,7 +1252,7 @@ __device__ __forceinline__ float block_sum(float x, float* red) {
   return t;
 }
 
-// W0 -> master weights, bf16 copy and row-norm targets (one block per row).
+// W0 -> master weights (if given), bf16 copy and row-norm targets (one block per row).
 __global__ void __launch_bounds__(ROW_THREADS) wide_prep_kernel(const float* __restrict__ w0, float* __restrict__ wm,
                                                                 __nv_bfloat16* __restrict__ wb, float* __restrict__ rho,
                                                                 int D, int F, int norm) {
@@ -1261,13 +1261,13 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_prep_kernel(const float* __r
   int len;
   row_geometry(blockIdx.x, D, F, off, len);
   ROW_CHECK(w0 + off, 4 * len);
-  ROW_CHECK(wm + off, 4 * len);
+  ROW_CHECK(wm ? wm + off : nullptr, 4 * len);
   ROW_CHECK(wb + off, 2 * len);
   ROW_CHECK(rho ? rho + blockIdx.x : nullptr, 4);
   float ss = 0.f;
   for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
     const float4 x = *reinterpret_cast<const float4*>(w0 + off + i);
-    *reinterpret_cast<float4*>(wm + off + i) = x;
+    if (wm) *reinterpret_cast<float4*>(wm + off + i) = x;
     *reinterpret_cast<uint2*>(wb + off + i) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
     ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
   }
@@ -1346,38 +1346,32 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_bprep_kernel(const float* __
   }
 }
 
-// Operands of one backward step: bf16 W (from w), bf16 -R (from r, if any),
-// and the adjoint accumulator lam = R (or 0).
-__global__ void wide_bstep_setup_kernel(const float* __restrict__ w, const float* __restrict__ r,
-                                        __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ nrb,
+// Operands of one backward step: bf16 W (from w) and, if lam is given, the adjoint
+// accumulator lam = 0 (a sequence without chunks).
+__global__ void wide_bstep_setup_kernel(const float* __restrict__ w, __nv_bfloat16* __restrict__ wb,
                                         float* __restrict__ lam, size_t P) {
   ROW_CHECK(w, 4 * P);
   ROW_CHECK(wb, 2 * P);
-  ROW_CHECK(r, 4 * P);
-  ROW_CHECK(r ? nrb : nullptr, 2 * P);
   ROW_CHECK(lam, 4 * P);
   for (size_t i = 4 * ((size_t)blockIdx.x * blockDim.x + threadIdx.x); i < P; i += 4 * (size_t)gridDim.x * blockDim.x) {
     const float4 x = *reinterpret_cast<const float4*>(w + i);
     *reinterpret_cast<uint2*>(wb + i) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
-    float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r) {
-      y = *reinterpret_cast<const float4*>(r + i);
-      *reinterpret_cast<uint2*>(nrb + i) = make_uint2(pack_bf16(-y.x, -y.y), pack_bf16(-y.z, -y.w));
-    }
-    *reinterpret_cast<float4*>(lam + i) = y;
+    if (lam) *reinterpret_cast<float4*>(lam + i) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
-// Closing a backward step (one block per row).  lam = dL/dW_j.  For j > 0 the
 // VJP of the row normalisation of update j-1 (W_j = rho w~ / max(|w~|, eps)):
 //   unclamped  R = (rho / |w~|) (lam - w_hat (w_hat . lam)),  clamped  R = (rho / eps) lam,
 //   w_hat = W_j / rho, drho += w_hat . lam;
+// R replaces lam (the next step adds its sums to it) and goes to nrb as bf16 -R
+// here, where it is in registers: at 12.6 M weights 37 us and a setup of 15, for
+// 36 and 28 when R went through memory to the setup kernel;
 // for j = 0, dW0 = lam + drho W0 / rho (added to dw0 when accumulate is set).
-__global__ void __launch_bounds__(ROW_THREADS) wide_bupdate_kernel(const float* __restrict__ lam,
+__global__ void __launch_bounds__(ROW_THREADS) wide_bupdate_kernel(float* __restrict__ lam,
                                                                    const float* __restrict__ wj,
                                                                    const float* __restrict__ wnorm,
                                                                    const float* __restrict__ rho, float* drho,
-                                                                   float* __restrict__ rout, const float* w0,
+                                                                   __nv_bfloat16* __restrict__ nrb, const float* w0,
                                                                    float* dw0, int accumulate, int D, int F, int norm,
                                                                    float eps) {
   __shared__ float red[ROW_THREADS / 32 + 1];
@@ -1391,7 +1385,7 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_bupdate_kernel(const float* 
     ROW_CHECK(dw0 + off, 4 * len);
     ROW_CHECK(norm == SCAL3R_NORM_ROW_W0 ? drho + blockIdx.x : nullptr, 4);
   } else {
-    ROW_CHECK(rout + off, 4 * len);
+    ROW_CHECK(nrb + off, 2 * len);
     if (norm != SCAL3R_NORM_NONE) {
       ROW_CHECK(wj + off, 4 * len);
       ROW_CHECK(wnorm + blockIdx.x, 4);
@@ -1414,24 +1408,35 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_bupdate_kernel(const float* 
     return;
   }
   if (norm == SCAL3R_NORM_NONE) {
-    for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS)
-      *reinterpret_cast<float4*>(rout + off + i) = *reinterpret_cast<const float4*>(lam + off + i);
+    for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
+      const float4 y = *reinterpret_cast<const float4*>(lam + off + i);
+      *reinterpret_cast<uint2*>(nrb + off + i) = make_uint2(pack_bf16(-y.x, -y.y), pack_bf16(-y.z, -y.w));
+    }
     return;
   }
   const float inv = rh > 0.f ? 1.f / rh : 0.f;
+  constexpr int kMaxPer = 4;   // float4 per thread, kept: one read of lam and W_j
+  float4 lv[kMaxPer], xv[kMaxPer];
   float pr = 0.f;
-  for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
-    const float4 l = *reinterpret_cast<const float4*>(lam + off + i);
-    const float4 x = *reinterpret_cast<const float4*>(wj + off + i);
-    pr += (x.x * l.x + x.y * l.y + x.z * l.z + x.w * l.w) * inv;
+#pragma unroll
+  for (int j = 0; j < kMaxPer; ++j) {
+    const int i = 4 * (threadIdx.x + j * ROW_THREADS);
+    if (i < len) {
+      const float4 l = lv[j] = *reinterpret_cast<const float4*>(lam + off + i);
+      const float4 x = xv[j] = *reinterpret_cast<const float4*>(wj + off + i);
+      // the rounding written out: the same sum however the loop is compiled
+      pr = fmaf(fmaf(x.w, l.w, fmaf(x.z, l.z, fmaf(x.x, l.x, __fmul_rn(x.y, l.y)))), inv, pr);
+    }
   }
   const float proj = block_sum(pr, red);
   const float n = wnorm[blockIdx.x];
   const bool clamped = !(n >= eps);
   const float c = clamped ? rh / eps : rh / n;
-  for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
-    const float4 l = *reinterpret_cast<const float4*>(lam + off + i);
-    const float4 x = *reinterpret_cast<const float4*>(wj + off + i);
+#pragma unroll
+  for (int j = 0; j < kMaxPer; ++j) {
+    const int i = 4 * (threadIdx.x + j * ROW_THREADS);
+    if (i >= len) break;
+    const float4 l = lv[j], x = xv[j];
     float4 y;
     if (clamped) {
       y = make_float4(c * l.x, c * l.y, c * l.z, c * l.w);
@@ -1439,7 +1444,8 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_bupdate_kernel(const float* 
       y = make_float4(c * (l.x - x.x * inv * proj), c * (l.y - x.y * inv * proj), c * (l.z - x.z * inv * proj),
                       c * (l.w - x.w * inv * proj));
     }
-    *reinterpret_cast<float4*>(rout + off + i) = y;
+    *reinterpret_cast<float4*>(lam + off + i) = y;
+    *reinterpret_cast<uint2*>(nrb + off + i) = make_uint2(pack_bf16(-y.x, -y.y), pack_bf16(-y.z, -y.w));
   }
   if (threadIdx.x == 0 && norm == SCAL3R_NORM_ROW_W0) drho[blockIdx.x] += proj;
 }
@@ -1509,7 +1515,7 @@ size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 struct WideBufs {
   __nv_bfloat16* act[8];
   float* wm;      // forward: master weights;  backward: lam (dL/dW_j)
-  float* gr;      // forward: chunk gradient;  backward: R (dL/dW~ of the next update)
+  float* gr;      // forward: chunk gradient;  backward: the adjoint, R (dL/dW~ of the next update) + its sums
   __nv_bfloat16* wb;    // bf16 weights
   __nv_bfloat16* nrb;   // backward: bf16 -R
   float* rho;
@@ -2311,14 +2317,20 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_gcs_update_kernel(const floa
   size_t off;
   int len;
   row_geometry(blockIdx.x, D, F, off, len);
+  constexpr int kMaxPer = 4;   // float4 per thread, kept: rows are at most 4 * 4 * ROW_THREADS long
+  float4 x[kMaxPer];
   float ss = 0.f, st = 0.f;
-  for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
-    const float4 a = *reinterpret_cast<const float4*>(w + off + i);
-    const float4 b = *reinterpret_cast<const float4*>(g + off + i);
-    const float4 t = *reinterpret_cast<const float4*>(w0 + off + i);
-    const float4 x = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-    ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
-    st += t.x * t.x + t.y * t.y + t.z * t.z + t.w * t.w;
+#pragma unroll
+  for (int j = 0; j < kMaxPer; ++j) {
+    const int i = 4 * (threadIdx.x + j * ROW_THREADS);
+    if (i < len) {
+      const float4 a = *reinterpret_cast<const float4*>(w + off + i);
+      const float4 b = *reinterpret_cast<const float4*>(g + off + i);
+      const float4 t = *reinterpret_cast<const float4*>(w0 + off + i);
+      x[j] = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+      ss += x[j].x * x[j].x + x[j].y * x[j].y + x[j].z * x[j].z + x[j].w * x[j].w;
+      st += t.x * t.x + t.y * t.y + t.z * t.z + t.w * t.w;
+    }
   }
   ss = block_sum(ss, red);
   st = block_sum(st, red);
@@ -2326,11 +2338,12 @@ __global__ void __launch_bounds__(ROW_THREADS) wide_gcs_update_kernel(const floa
   const float rho = (norm == SCAL3R_NORM_UNIT) ? 1.f : sqrtf(st);
   const float scale = (norm == SCAL3R_NORM_NONE) ? 1.f : rho / fmaxf(n, eps);
   if (threadIdx.x == 0 && wnorm) wnorm[blockIdx.x] = n;
-  for (int i = 4 * threadIdx.x; i < len; i += 4 * ROW_THREADS) {
-    const float4 a = *reinterpret_cast<const float4*>(w + off + i);
-    const float4 b = *reinterpret_cast<const float4*>(g + off + i);
-    *reinterpret_cast<float4*>(w_out + off + i) =
-        make_float4((a.x - b.x) * scale, (a.y - b.y) * scale, (a.z - b.z) * scale, (a.w - b.w) * scale);
+#pragma unroll
+  for (int j = 0; j < kMaxPer; ++j) {
+    const int i = 4 * (threadIdx.x + j * ROW_THREADS);
+    if (i < len)
+      *reinterpret_cast<float4*>(w_out + off + i) =
+          make_float4(x[j].x * scale, x[j].y * scale, x[j].z * scale, x[j].w * scale);
   }
 }
 
@@ -2354,7 +2367,7 @@ cudaError_t wide_partial_grad(const Plan& pl, const Shape& sh, const Params& prm
       }
       const float* wsrc = prm.w0 + (size_t)s * prm.w0_seq_stride + (size_t)h * P;
       WIDE_TRY(launch(1, 0, 0, [&] {
-        wide_prep_kernel<<<R, ROW_THREADS, 0, st>>>(wsrc, w.wm, w.wb, nullptr, D, F, prm.norm);
+        wide_prep_kernel<<<R, ROW_THREADS, 0, st>>>(wsrc, nullptr, w.wb, nullptr, D, F, prm.norm);
         return cudaGetLastError();
       }));
       WIDE_TRY(key_grad(cx, h, c0, w.wb, gout, w.act, w.ex, w.spl));
@@ -2396,7 +2409,7 @@ cudaError_t wide_apply(const Plan& pl, const Shape& sh, const Params& prm, void*
       if (c1 == c0) continue;
       const float* wsrc = prm.w0 + (size_t)s * prm.w0_seq_stride + (size_t)h * P;
       WIDE_TRY(launch(1, 0, 0, [&] {
-        wide_prep_kernel<<<R, ROW_THREADS, 0, st>>>(wsrc, w.wm, w.wb, nullptr, D, F, prm.norm);
+        wide_prep_kernel<<<R, ROW_THREADS, 0, st>>>(wsrc, nullptr, w.wb, nullptr, D, F, prm.norm);
         return cudaGetLastError();
       }));
       WIDE_TRY(apply_chunk(cx, h, c0, w.wb, w.act[0]));
@@ -2546,7 +2559,7 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
   const size_t FD = (size_t)F * D;
   const __nv_bfloat16 *w1 = w.wb, *w3 = w.wb + FD, *w2 = w.wb + 2 * FD;
   const __nv_bfloat16 *r1 = w.nrb, *r3 = w.nrb + FD, *r2 = w.nrb + 2 * FD;   // -R
-  float *lam1 = w.wm, *lam3 = w.wm + FD, *lam2 = w.wm + 2 * FD;
+  float *lam1 = w.gr, *lam3 = w.gr + FD, *lam2 = w.gr + 2 * FD;
   const int nparts = deta_parts(sh, prm.lr_mat);
   for (int s = 0; s < pl.S; ++s) {
     for (int h = 0; h < H; ++h) {
@@ -2578,8 +2591,10 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
       for (int j = j1; j >= j0; --j) {
         const float* wj = (j == j0) ? wbase : w.seg + (size_t)(j - j0 - 1) * P;
         const bool key = j < n;
+        // the last chunk's step has no R: its sums are stored, not added to zeros
+        const bool fresh = !key && n > 0;
         WIDE_TRY(launch(1, 0, 0, [&] {
-          wide_bstep_setup_kernel<<<4 * num_sms(), 256, 0, st>>>(wj, key ? w.gr : nullptr, w.wb, w.nrb, w.wm, P);
+          wide_bstep_setup_kernel<<<4 * num_sms(), 256, 0, st>>>(wj, w.wb, n == 0 ? w.gr : nullptr, P);
           return cudaGetLastError();
         }));
         if (j >= 1) {   // apply VJP of chunk j-1
@@ -2618,13 +2633,13 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
             GemmArgs& a = l[1 + i];
             WIDE_MAP(mat_map(&a.a[0], i ? dz3 : dz1, M, F, 64) && tok_map(&a.b[0], prm.q, T, H, D, 64));
             a.M = F; a.N = D; a.K = M; a.a_mn = 1; a.b_mn = 1; a.hb = h; a.yb = (int)t0;
-            a.epi = EPI_F32_ADD; a.out[0] = i ? lam3 : lam1; a.ld_out = D;
+            a.epi = fresh ? EPI_F32 : EPI_F32_ADD; a.out[0] = i ? lam3 : lam1; a.ld_out = D;
           }
           {   // lam2 += d_O^T uq
             GemmArgs& a = l[3];
             WIDE_MAP(tok_map(&a.a[0], prm.d_o, T, H, D, 64) && mat_map(&a.b[0], uq, M, F, 64));
             a.M = D; a.N = F; a.K = M; a.a_mn = 1; a.b_mn = 1; a.ha = h; a.ya = (int)t0;
-            a.epi = EPI_F32_ADD; a.out[0] = lam2; a.ld_out = F;
+            a.epi = fresh ? EPI_F32 : EPI_F32_ADD; a.out[0] = lam2; a.ld_out = F;
           }
           WIDE_TRY(run_gemm_list(cx, l, fl, 4, w.spl));
         }
@@ -2700,7 +2715,7 @@ cudaError_t wide_backward(const Plan& pl, const Shape& sh, const Params& prm, in
         // normalisation VJP of update j-1 -> R, or dW0
         const float* wn = (j >= 1) ? prm.wnorm_in + ((size_t)(c0 + j - 1) * H + h) * R : nullptr;
         WIDE_TRY(launch(1, 0, 0, [&] {
-          wide_bupdate_kernel<<<R, ROW_THREADS, 0, st>>>(w.wm, wj, wn, w.rho, w.drho, w.gr, w0,
+          wide_bupdate_kernel<<<R, ROW_THREADS, 0, st>>>(w.gr, wj, wn, w.rho, w.drho, w.nrb, w0,
                                                          j == 0 ? dw0 : nullptr, acc_dw0 ? 1 : 0, D, F, prm.norm,
                                                          prm.eps);
           return cudaGetLastError();
