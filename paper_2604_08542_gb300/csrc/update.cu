@@ -69,19 +69,31 @@ __device__ __forceinline__ float4 add4(float4 a, float4 b) {
 __device__ __forceinline__ float4 scale4(float4 a, float s) { return make_float4(a.x * s, a.y * s, a.z * s, a.w * s); }
 __device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 
-// The sum of squares of four elements with its rounding written out: a row's
-// target is formed from w0 by several kernels, which have to agree to the bit
-// (the backward's recomputed weights are the forward's).
-__device__ __forceinline__ float sumsq4(float4 a) {
-  return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.x, a.x, __fmul_rn(a.y, a.y))));
+// Dot products with their rounding written out: a row's norm, its target and its
+// adjoint's projection are formed by several kernels, which have to agree to the
+// bit (the backward's recomputed weights are the forward's).
+__device__ __forceinline__ float rdot4(float4 a, float4 b) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.x, b.x, __fmul_rn(a.y, b.y))));
+}
+__device__ __forceinline__ float sumsq4(float4 a) { return rdot4(a, a); }   // of w0: the target
+__device__ __forceinline__ float normsq4(float4 a) {                        // of the updated row
+  return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.y, a.y, __fmul_rn(a.x, a.x))));
 }
 
+// The two update kernels exist twice.  A grid whose blocks are all resident at
+// three a SM (16 chains of the (64, 128) layer: 384 blocks) waits for memory
+// round trips only, and takes its slots eight at a time (80 registers).  A
+// larger one needs warps in flight: two slots at a time, so that eight blocks
+// (the backward's: six) fit a SM.  The update of 352 chains took 38 us with the
+// first form and takes 24.5 (at 100 MB, 4.2 TB/s), of 32 chains 6.8 and 6.0.
+constexpr int kFewBlocks = 3, kManyBlocks = 8, kManyBlocksBwd = 6;
+
 // x + the slots slot0 .. slot0 + n - 1 at element offset `off`, added one by
-// one in slot order (fixed-order reduction); the loads of a batch of eight
+// one in slot order (fixed-order reduction); the loads of a batch of kBatch
 // slots are issued before any of them is added, so the sum costs one memory
-// round trip per eight slots rather than one per slot.
+// round trip per batch rather than one per slot.
+template <int kBatch>
 __device__ __forceinline__ float4 add_slots(float4 x, const float* part, int slot0, int n, size_t P, size_t off) {
-  constexpr int kBatch = 8;
   for (int b = 0; b < n; b += kBatch) {
     float4 v[kBatch];
 #pragma unroll
@@ -120,36 +132,39 @@ __global__ void prep_kernel(Params p) {
 // Forward update of one chain at step `step`:
 //   W~ = W_step + sum_slots partial (fixed slot order),
 //   W_{step+1} row = W~ row * rho / max(||W~ row||, eps).
-// With w_items (a forward's first step) W_step is w0 itself and the row targets
+// FIRST (a forward's first step): W_step is w0 itself and the row targets
 // come from it here, so that no launch copies w0 first (3.6 us and its launch on
 // every forward call).
-__global__ void update_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
+template <bool FIRST, int kBatch>
+__global__ void __launch_bounds__(kThreads, kBatch == 8 ? kFewBlocks : kManyBlocks)
+update_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
   pdl_wait();
   const UpdateItem u = upd[blockIdx.x];
   const RowSlice s = row_slice(blockIdx.y, p.D, p.F);
   const int P = 3 * p.F * p.D, R = 2 * p.F + p.D;
   const int chains = p.S * p.H;
   const int h = u.chain % p.H;
-  const float* wcur = p.w_items ? chain_w0(p, u.chain) : p.wm + ((size_t)(step & 1) * chains + u.chain) * P;
+  const float* wcur = FIRST ? chain_w0(p, u.chain) : p.wm + ((size_t)(step & 1) * chains + u.chain) * P;
   float* wnext = p.wm + ((size_t)((step + 1) & 1) * chains + u.chain) * P;
   if (u.chunk < 0) {   // sequence without chunks: w_final = w0
     if (p.w_final && s.valid) st4(p.w_final + ((size_t)u.seq * p.H + h) * P + s.off, ld4(wcur + s.off));
     return;
   }
-  float4 x = make_float4(0.f, 0.f, 0.f, 0.f), w0 = x;
-  float rho = 1.f;
+  float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+  float rho = 1.f, ss0 = 0.f;
   if (s.valid) {
     // the row target is loaded before the slot sum so that its round trip
     // overlaps the sum's
-    if (p.norm != SCAL3R_NORM_NONE && !p.w_items) rho = ld_chk(p.rho + (size_t)u.chain * R + s.r);
-    w0 = ld4(wcur + s.off);
-    x = add_slots(w0, p.part, u.slot0, u.nslots, P, s.off);
+    if (p.norm != SCAL3R_NORM_NONE && !FIRST) rho = ld_chk(p.rho + (size_t)u.chain * R + s.r);
+    x = ld4(wcur + s.off);
+    if (FIRST) ss0 = sumsq4(x);
+    x = add_slots<kBatch>(x, p.part, u.slot0, u.nslots, P, s.off);
   }
-  if (p.w_items && p.norm != SCAL3R_NORM_NONE) {   // the chain's first update: the row targets, kept for the next ones
-    rho = row_target(p, group_sum(sumsq4(w0), s.group));
+  if (FIRST && p.norm != SCAL3R_NORM_NONE) {   // the chain's first update: the row targets, kept for the next ones
+    rho = row_target(p, group_sum(ss0, s.group));
     if (s.valid && s.c4 == 0) st_chk(p.rho + (size_t)u.chain * R + s.r, rho);
   }
-  const float n = sqrtf(group_sum(dot4(x, x), s.group));
+  const float n = sqrtf(group_sum(normsq4(x), s.group));
   if (!s.valid) return;
   float scale = 1.f;
   if (p.norm != SCAL3R_NORM_NONE) scale = rho / fmaxf(n, p.eps);
@@ -184,7 +199,9 @@ __global__ void bprep_kernel(Params p) {
 //   W_row = rho w~ / max(||w~||, eps), w_hat = W_row / rho:
 //   unclamped  R = (rho / ||w~||) (lambda - w_hat (w_hat . lambda))
 //   clamped    R = (rho / eps) lambda;      drho += w_hat . lambda in both
-__global__ void bupdate_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
+template <int kBatch>
+__global__ void __launch_bounds__(kThreads, kBatch == 8 ? kFewBlocks : kManyBlocksBwd)
+bupdate_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
   pdl_wait();
   (void)step;
   const UpdateItem u = upd[blockIdx.x];
@@ -208,7 +225,7 @@ __global__ void bupdate_kernel(Params p, const UpdateItem* __restrict__ upd, int
       n = ld_chk(p.wnorm_in + ((size_t)u.chunk * p.H + h) * R + s.r);
     }
     if (!u.last) lam = ld4(rb + s.off);
-    lam = add_slots(lam, p.part, u.slot0, u.nslots, P, s.off);
+    lam = add_slots<kBatch>(lam, p.part, u.slot0, u.nslots, P, s.off);
   }
   if (u.first) {
     if (!s.valid) return;
@@ -224,7 +241,7 @@ __global__ void bupdate_kernel(Params p, const UpdateItem* __restrict__ upd, int
   }
   const float inv_rho = rho > 0.f ? 1.f / rho : 0.f;
   const float4 what = scale4(wck, inv_rho);
-  const float proj = group_sum(dot4(what, lam), s.group);
+  const float proj = group_sum(rdot4(what, lam), s.group);
   if (!s.valid) return;
   float4 out;
   if (!(n >= p.eps)) {
@@ -273,7 +290,7 @@ __global__ void gsum_kernel(Params p, const UpdateItem* __restrict__ upd, float*
   const int P = 3 * p.F * p.D;
   const int h = u.chain % p.H;
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (u.chunk >= 0) x = add_slots(x, p.part, u.slot0, u.nslots, P, s.off);
+  if (u.chunk >= 0) x = add_slots<8>(x, p.part, u.slot0, u.nslots, P, s.off);
   st4(grad + ((size_t)u.seq * p.H + h) * P + s.off, scale4(x, -1.f));
 }
 
@@ -358,6 +375,16 @@ __global__ void gcs_update_kernel(Params p, const float* w, int64_t w_stride, co
 
 int row_blocks(const Params& p) { return (2 * p.F * p.D + 1023) / 1024 + (p.F * p.D + 1023) / 1024; }
 
+bool few_blocks(int blocks) {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  }();
+  return blocks <= kFewBlocks * sms;
+}
+
 }  // namespace
 
 // Shapes the row kernels handle: D/4 and F/4 powers of two dividing 32.
@@ -373,12 +400,16 @@ cudaError_t launch_prep(const Params& prm, int chains, cudaStream_t st) {
 
 cudaError_t launch_update(const Params& prm, const UpdateItem* upd, int nupd, int step, cudaStream_t st) {
   if (nupd == 0) return cudaSuccess;
-  return launch_pdl(update_kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
+  const bool few = few_blocks(nupd * row_blocks(prm));
+  auto kernel = prm.w_items ? (few ? update_kernel<true, 8> : update_kernel<true, 2>)
+                            : (few ? update_kernel<false, 8> : update_kernel<false, 2>);
+  return launch_pdl(kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
 }
 
 cudaError_t launch_bupdate(const Params& prm, const UpdateItem* upd, int nupd, int step, cudaStream_t st) {
   if (nupd == 0) return cudaSuccess;
-  return launch_pdl(bupdate_kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
+  auto kernel = few_blocks(nupd * row_blocks(prm)) ? bupdate_kernel<8> : bupdate_kernel<2>;
+  return launch_pdl(kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
 }
 
 cudaError_t launch_bprep(const Params& prm, int chains, cudaStream_t st);
