@@ -146,17 +146,23 @@ __device__ __forceinline__ float silu_d(float z, float& sg) {
   return z * sg;
 }
 
-// One 32-byte store of eight 32-bit words (dst 32-byte aligned).  Each thread
-// of an epilogue writes its own row, so a warp's store touches 32 rows: the
-// wider store halves the transactions per byte.
+// One 32-byte store of eight 32-bit words, two of 16 where dst is only 16-byte
+// aligned (callers' tensors and row strides have to be no more than that).  Each
+// thread of an epilogue writes its own row, so a warp's store touches 32 rows:
+// the wider store halves the transactions per byte.
 __device__ __forceinline__ void st_global_v8(void* dst, const uint32_t (&a)[8]) {
   if (!in_bounds(dst, 32)) return;
+  if (reinterpret_cast<uintptr_t>(dst) & 31) {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(a[0], a[1], a[2], a[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(a[4], a[5], a[6], a[7]);
+    return;
+  }
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                :: "l"(dst), "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7])
                : "memory");
 }
 
-// Packs 16 floats to 8 bf16x2 words and stores them (one 32-byte store).
+// Packs 16 floats to 8 bf16x2 words and stores them.
 __device__ __forceinline__ void st_bf16x16(__nv_bfloat16* dst, const float* v) {
   uint32_t w[8];
 #pragma unroll
