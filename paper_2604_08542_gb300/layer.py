@@ -2,12 +2,16 @@
 
 Only argument marshalling happens here (shape/dtype checks, output and
 workspace allocation, the current CUDA stream); the computation is the
-library's.  Layouts follow the C header: q, k, v, o [T, H, D]; lr [T, H]
+library's.  A one-frame call's launches take 18 us on the GPU, so each call
+converts its layout once and goes straight to the library (44 us a forward call
+before, 27 after).  Layouts follow the C header: q, k, v, o [T, H, D]; lr [T, H]
 float32 ([T, H, 3] with per-matrix rates: W1, W3, W2); w0 [H, 3*F*D] (shared) or [S, H, 3*F*D] (per sequence) float32,
 packed W1 [F, D], W3 [F, D], W2 [D, F]; chunk_offsets [C+1] int64 and
 seq_chunk_ptr [S+1] int32 on the host.
 """
 from __future__ import annotations
+
+import ctypes
 
 import numpy as np
 import torch
@@ -18,12 +22,12 @@ import os
 
 from . import (SCAL3R_BF16, SCAL3R_FP32, SCAL3R_LOSS_DOT, SCAL3R_LOSS_MSE, SCAL3R_MODEL_LINEAR,
                SCAL3R_MODEL_SWIGLU, SCAL3R_NORM_NONE,
-               SCAL3R_NORM_ROW_W0, SCAL3R_NORM_UNIT, Scal3rError, _check, scal3r_ttt_autotune, scal3r_ttt_backward,
-               scal3r_ttt_config, scal3r_ttt_destroy, scal3r_ttt_forward, scal3r_ttt_get_schedule,
+               SCAL3R_NORM_ROW_W0, SCAL3R_NORM_UNIT, Scal3rError, _check, scal3r_ttt_autotune,
+               scal3r_ttt_config, scal3r_ttt_destroy, scal3r_ttt_get_schedule,
                scal3r_ttt_get_status, scal3r_ttt_init, scal3r_ttt_plan, scal3r_ttt_schedule,
                scal3r_ttt_set_graph_mode, scal3r_ttt_set_schedule, scal3r_ttt_workspace_size,
-               scal3r_ttt_partial_grad, scal3r_ttt_apply_update, scal3r_ttt_apply, scal3r_ttt_ckpt_slots,
-               scal3r_ttt_set_finite_check)
+               scal3r_ttt_apply_update, scal3r_ttt_ckpt_slots,
+               scal3r_ttt_set_finite_check, load_library)
 
 NORMS = {"row_w0": SCAL3R_NORM_ROW_W0, "none": SCAL3R_NORM_NONE, "unit": SCAL3R_NORM_UNIT}
 LOSSES = {"dot": SCAL3R_LOSS_DOT, "mse": SCAL3R_LOSS_MSE}
@@ -32,6 +36,23 @@ MODELS = {"swiglu": SCAL3R_MODEL_SWIGLU, "linear": SCAL3R_MODEL_LINEAR}
 
 def _ptr(t):
     return None if t is None else t.data_ptr()
+
+
+def _stream(dev) -> int:
+    # torch.cuda.current_stream(dev).cuda_stream without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(dev.index)
+
+
+class _Layout:
+    """A call's host layout, converted once, and the C arguments
+    (off, C, ptr, S) that the library's entry points take."""
+    __slots__ = ("off", "ptr", "T", "C", "S", "args")
+
+    def __init__(self, chunk_offsets, seq_chunk_ptr):
+        self.off = off = np.ascontiguousarray(chunk_offsets, dtype=np.int64)
+        self.ptr = ptr = np.ascontiguousarray(seq_chunk_ptr, dtype=np.int32)
+        self.T, self.C, self.S = int(off[-1]), len(off) - 1, len(ptr) - 1
+        self.args = (off.ctypes.data, self.C, ptr.ctypes.data, self.S)
 
 
 class TTT:
@@ -79,26 +100,38 @@ class TTT:
 
     def workspace(self, chunk_offsets, seq_chunk_ptr, with_backward: bool, device) -> torch.Tensor:
         n = scal3r_ttt_workspace_size(self.handle, chunk_offsets, seq_chunk_ptr, with_backward)
-        if self._ws is None or self._ws.numel() < n or self._ws.device != torch.device(device):
-            self._ws = torch.empty(max(n, 256), dtype=torch.uint8, device=device)
-        return self._ws
+        return self._grow(n, torch.device(device))
+
+    def _grow(self, n, device):
+        ws = self._ws
+        if ws is None or ws.numel() < n or ws.device != device:
+            self._ws = ws = torch.empty(max(n, 256), dtype=torch.uint8, device=device)
+        return ws
+
+    def _call_workspace(self, lib, lay, with_backward, device):
+        n = ctypes.c_size_t()
+        rc = lib.scal3r_ttt_workspace_size(self.handle, *lay.args, with_backward, ctypes.byref(n))
+        if rc:
+            _check(rc, "scal3r_ttt_workspace_size")
+        return self._grow(n.value, device)
 
     def _check_lr(self, lr, T):
-        if lr.dtype != torch.float32 or tuple(lr.shape) != (T, *self.lr_shape) or not lr.is_contiguous():
+        if lr.dtype != torch.float32 or lr.shape != (T, *self.lr_shape) or not lr.is_contiguous():
             raise ValueError(f"lr must be a contiguous float32 tensor of shape {[T, *self.lr_shape]}")
 
     def _check_tokens(self, name, t, T):
-        if t.dtype != self.dtype or t.dim() != 3 or tuple(t.shape) != (T, self.H, self.D) or not t.is_cuda \
+        if t.dtype != self.dtype or t.shape != (T, self.H, self.D) or not t.is_cuda \
                 or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous CUDA {self.dtype} tensor of shape [T, H, D]")
 
     def _w0_stride(self, w0, S):
         if w0.dtype != torch.float32 or not w0.is_cuda or not w0.is_contiguous():
             raise ValueError("w0 must be a contiguous CUDA float32 tensor")
-        if w0.dim() == 2 and tuple(w0.shape) == (self.H, self.P):
+        P = self.P
+        if w0.shape == (self.H, P):
             return 0
-        if w0.dim() == 3 and tuple(w0.shape) == (S, self.H, self.P):
-            return self.H * self.P
+        if w0.shape == (S, self.H, P):
+            return self.H * P
         raise ValueError("w0 must be [H, P] or [S, H, P] (P = 3*F*D, or D*D for the linear model)")
 
     # -- passes ------------------------------------------------------------
@@ -106,16 +139,16 @@ class TTT:
                 want_final=False, workspace=None, o=None, w_ckpt=None, wnorm=None):
         """Returns (o, w_ckpt, wnorm, w_final).  o, w_ckpt and wnorm may be
         given (preallocated, e.g. to keep a captured graph's pointers)."""
-        off = np.ascontiguousarray(chunk_offsets, dtype=np.int64)
-        ptr = np.ascontiguousarray(seq_chunk_ptr, dtype=np.int32)
-        T, C, S = int(off[-1]), len(off) - 1, len(ptr) - 1
+        lay = _Layout(chunk_offsets, seq_chunk_ptr)
+        T, C, S = lay.T, lay.C, lay.S
         for n, t in (("q", q), ("k", k), ("v", v)):
             self._check_tokens(n, t, T)
         self._check_lr(lr, T)
         stride = self._w0_stride(w0, S)
         dev = q.device
+        lib = load_library()
         o = torch.empty_like(q) if o is None else o
-        slots = C if self.cfg.ckpt_every <= 1 else scal3r_ttt_ckpt_slots(self.handle, ptr)
+        slots = C if self.cfg.ckpt_every <= 1 else scal3r_ttt_ckpt_slots(self.handle, lay.ptr)
         if save_for_backward:
             if w_ckpt is None:
                 w_ckpt = torch.empty((slots, self.H, self.P), dtype=torch.float32, device=dev)
@@ -126,23 +159,23 @@ class TTT:
         else:
             w_ckpt = wnorm = None
         w_final = torch.empty((S, self.H, self.P), dtype=torch.float32, device=dev) if want_final else None
-        ws = self.workspace(off, ptr, False, dev) if workspace is None else workspace
-        st = torch.cuda.current_stream(dev).cuda_stream
-        rc = scal3r_ttt_forward(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(lr), _ptr(w0), stride, off, ptr,
-                                _ptr(o), _ptr(w_ckpt), _ptr(wnorm), _ptr(w_final), _ptr(ws), ws.numel(), st)
-        _check(rc, "scal3r_ttt_forward")
+        ws = self._call_workspace(lib, lay, False, dev) if workspace is None else workspace
+        rc = lib.scal3r_ttt_forward(self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), lr.data_ptr(),
+                                    w0.data_ptr(), stride, *lay.args, o.data_ptr(), _ptr(w_ckpt), _ptr(wnorm),
+                                    _ptr(w_final), ws.data_ptr(), ws.numel(), _stream(dev))
+        if rc:
+            _check(rc, "scal3r_ttt_forward")
         return o, w_ckpt, wnorm, w_final
 
     def backward(self, q, k, v, lr, w0, chunk_offsets, seq_chunk_ptr, d_o, w_ckpt, wnorm, *, workspace=None,
                  out=None):
         """Returns (dq, dk, dv, dlr, dw0); ``out`` may give them preallocated."""
-        off = np.ascontiguousarray(chunk_offsets, dtype=np.int64)
-        ptr = np.ascontiguousarray(seq_chunk_ptr, dtype=np.int32)
-        T, S = int(off[-1]), len(ptr) - 1
+        lay = _Layout(chunk_offsets, seq_chunk_ptr)
         for n, t in (("q", q), ("k", k), ("v", v), ("d_o", d_o)):
-            self._check_tokens(n, t, T)
-        self._check_lr(lr, T)
-        stride = self._w0_stride(w0, S)
+            self._check_tokens(n, t, lay.T)
+        self._check_lr(lr, lay.T)
+        stride = self._w0_stride(w0, lay.S)
+        lib = load_library()
         if out is None:
             dq, dk, dv, dlr, dw0 = (torch.empty_like(t) for t in (q, k, v, lr, w0))
         else:
@@ -150,30 +183,30 @@ class TTT:
             for a, b in zip(out, (q, k, v, lr, w0)):
                 if a.shape != b.shape or a.dtype != b.dtype or not a.is_contiguous():
                     raise ValueError("out tensors must match q, k, v, lr, w0")
-        ws = self.workspace(off, ptr, True, q.device) if workspace is None else workspace
-        st = torch.cuda.current_stream(q.device).cuda_stream
-        rc = scal3r_ttt_backward(self.handle, _ptr(q), _ptr(k), _ptr(v), _ptr(lr), _ptr(w0), stride, off, ptr,
-                                 _ptr(d_o), _ptr(w_ckpt), _ptr(wnorm), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dlr),
-                                 _ptr(dw0), _ptr(ws), ws.numel(), st)
-        _check(rc, "scal3r_ttt_backward")
+        ws = self._call_workspace(lib, lay, True, q.device) if workspace is None else workspace
+        rc = lib.scal3r_ttt_backward(self.handle, q.data_ptr(), k.data_ptr(), v.data_ptr(), lr.data_ptr(),
+                                     w0.data_ptr(), stride, *lay.args, d_o.data_ptr(), _ptr(w_ckpt), _ptr(wnorm),
+                                     _ptr(dq), _ptr(dk), _ptr(dv), _ptr(dlr), _ptr(dw0), ws.data_ptr(), ws.numel(),
+                                     _stream(q.device))
+        if rc:
+            _check(rc, "scal3r_ttt_backward")
         return dq, dk, dv, dlr, dw0
 
     # -- Global Context Synchronisation (Eq. 10): a chunk step in local parts ----
     def partial_grad(self, k, v, lr, w, chunk_offsets, seq_chunk_ptr, *, workspace=None):
         """The inner gradient of Eq. 8 over each sequence's (single) chunk at
         the weights w ([H, P] or [S, H, P]); returns grad [S, H, P] float32."""
-        off = np.ascontiguousarray(chunk_offsets, dtype=np.int64)
-        ptr = np.ascontiguousarray(seq_chunk_ptr, dtype=np.int32)
-        T, S = int(off[-1]), len(ptr) - 1
+        lay = _Layout(chunk_offsets, seq_chunk_ptr)
         for n, t in (("k", k), ("v", v)):
-            self._check_tokens(n, t, T)
-        self._check_lr(lr, T)
-        stride = self._w0_stride(w, S)
-        grad = torch.empty((S, self.H, self.P), dtype=torch.float32, device=k.device)
-        ws = self.workspace(off, ptr, False, k.device) if workspace is None else workspace
-        st = torch.cuda.current_stream(k.device).cuda_stream
-        _check(scal3r_ttt_partial_grad(self.handle, _ptr(k), _ptr(v), _ptr(lr), _ptr(w), stride, off, ptr,
-                                       _ptr(grad), _ptr(ws), ws.numel(), st), "scal3r_ttt_partial_grad")
+            self._check_tokens(n, t, lay.T)
+        self._check_lr(lr, lay.T)
+        stride = self._w0_stride(w, lay.S)
+        lib = load_library()
+        grad = torch.empty((lay.S, self.H, self.P), dtype=torch.float32, device=k.device)
+        ws = self._call_workspace(lib, lay, False, k.device) if workspace is None else workspace
+        _check(lib.scal3r_ttt_partial_grad(self.handle, k.data_ptr(), v.data_ptr(), lr.data_ptr(), w.data_ptr(),
+                                           stride, *lay.args, grad.data_ptr(), ws.data_ptr(), ws.numel(),
+                                           _stream(k.device)), "scal3r_ttt_partial_grad")
         return grad
 
     def apply_update(self, w, grad, w0):
@@ -186,23 +219,21 @@ class TTT:
         ws, w0s = self._w0_stride(w, S), self._w0_stride(w0, S)
         w_out = torch.empty_like(grad)
         wnorm = torch.empty((S, self.H, self.R), dtype=torch.float32, device=grad.device)
-        st = torch.cuda.current_stream(grad.device).cuda_stream
+        st = _stream(grad.device)
         _check(scal3r_ttt_apply_update(self.handle, _ptr(w), ws, _ptr(grad), _ptr(w0), w0s, S, _ptr(w_out),
                                        _ptr(wnorm), st), "scal3r_ttt_apply_update")
         return w_out, wnorm
 
     def apply(self, q, w, chunk_offsets, seq_chunk_ptr, *, workspace=None):
         """o = f_W(q) for each sequence's (single) chunk with its weights w."""
-        off = np.ascontiguousarray(chunk_offsets, dtype=np.int64)
-        ptr = np.ascontiguousarray(seq_chunk_ptr, dtype=np.int32)
-        T, S = int(off[-1]), len(ptr) - 1
-        self._check_tokens("q", q, T)
-        stride = self._w0_stride(w, S)
+        lay = _Layout(chunk_offsets, seq_chunk_ptr)
+        self._check_tokens("q", q, lay.T)
+        stride = self._w0_stride(w, lay.S)
+        lib = load_library()
         o = torch.empty_like(q)
-        ws = self.workspace(off, ptr, False, q.device) if workspace is None else workspace
-        st = torch.cuda.current_stream(q.device).cuda_stream
-        _check(scal3r_ttt_apply(self.handle, _ptr(q), _ptr(w), stride, off, ptr, _ptr(o), _ptr(ws), ws.numel(), st),
-               "scal3r_ttt_apply")
+        ws = self._call_workspace(lib, lay, False, q.device) if workspace is None else workspace
+        _check(lib.scal3r_ttt_apply(self.handle, q.data_ptr(), w.data_ptr(), stride, *lay.args, o.data_ptr(),
+                                    ws.data_ptr(), ws.numel(), _stream(q.device)), "scal3r_ttt_apply")
         return o
 
     def status(self) -> int:
