@@ -82,10 +82,12 @@ __device__ __forceinline__ float normsq4(float4 a) {                        // o
 
 // The two update kernels exist twice.  A grid whose blocks are all resident at
 // three a SM (16 chains of the (64, 128) layer: 384 blocks) waits for memory
-// round trips only, and takes its slots eight at a time (80 registers).  A
-// larger one needs warps in flight: two slots at a time, so that eight blocks
-// (the backward's: six) fit a SM.  The update of 352 chains took 38 us with the
-// first form and takes 24.5 (at 100 MB, 4.2 TB/s), of 32 chains 6.8 and 6.0.
+// round trips only, and takes its slots six at a time in 70 to 78 registers
+// (eight at a time spill, 0.4 % of a 256-frame training step).  A larger one
+// needs warps in flight: two slots at a time, so that eight blocks (the
+// backward's: six) fit a SM.  The update of 352 chains took 38 us with eight at a
+// time and takes 24.5 (at 100 MB, 4.2 TB/s), of 32 chains 6.8 and 6.0.
+constexpr int kFewSlots = 6, kManySlots = 2;
 constexpr int kFewBlocks = 3, kManyBlocks = 8, kManyBlocksBwd = 6;
 
 // x + the slots slot0 .. slot0 + n - 1 at element offset `off`, added one by
@@ -136,7 +138,7 @@ __global__ void prep_kernel(Params p) {
 // come from it here, so that no launch copies w0 first (3.6 us and its launch on
 // every forward call).
 template <bool FIRST, int kBatch>
-__global__ void __launch_bounds__(kThreads, kBatch == 8 ? kFewBlocks : kManyBlocks)
+__global__ void __launch_bounds__(kThreads, kBatch == kFewSlots ? kFewBlocks : kManyBlocks)
 update_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
   pdl_wait();
   const UpdateItem u = upd[blockIdx.x];
@@ -200,7 +202,7 @@ __global__ void bprep_kernel(Params p) {
 //   unclamped  R = (rho / ||w~||) (lambda - w_hat (w_hat . lambda))
 //   clamped    R = (rho / eps) lambda;      drho += w_hat . lambda in both
 template <int kBatch>
-__global__ void __launch_bounds__(kThreads, kBatch == 8 ? kFewBlocks : kManyBlocksBwd)
+__global__ void __launch_bounds__(kThreads, kBatch == kFewSlots ? kFewBlocks : kManyBlocksBwd)
 bupdate_kernel(Params p, const UpdateItem* __restrict__ upd, int step) {
   pdl_wait();
   (void)step;
@@ -290,7 +292,7 @@ __global__ void gsum_kernel(Params p, const UpdateItem* __restrict__ upd, float*
   const int P = 3 * p.F * p.D;
   const int h = u.chain % p.H;
   float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (u.chunk >= 0) x = add_slots<8>(x, p.part, u.slot0, u.nslots, P, s.off);
+  if (u.chunk >= 0) x = add_slots<kFewSlots>(x, p.part, u.slot0, u.nslots, P, s.off);
   st4(grad + ((size_t)u.seq * p.H + h) * P + s.off, scale4(x, -1.f));
 }
 
@@ -401,14 +403,14 @@ cudaError_t launch_prep(const Params& prm, int chains, cudaStream_t st) {
 cudaError_t launch_update(const Params& prm, const UpdateItem* upd, int nupd, int step, cudaStream_t st) {
   if (nupd == 0) return cudaSuccess;
   const bool few = few_blocks(nupd * row_blocks(prm));
-  auto kernel = prm.w_items ? (few ? update_kernel<true, 8> : update_kernel<true, 2>)
-                            : (few ? update_kernel<false, 8> : update_kernel<false, 2>);
+  auto kernel = prm.w_items ? (few ? update_kernel<true, kFewSlots> : update_kernel<true, kManySlots>)
+                            : (few ? update_kernel<false, kFewSlots> : update_kernel<false, kManySlots>);
   return launch_pdl(kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
 }
 
 cudaError_t launch_bupdate(const Params& prm, const UpdateItem* upd, int nupd, int step, cudaStream_t st) {
   if (nupd == 0) return cudaSuccess;
-  auto kernel = few_blocks(nupd * row_blocks(prm)) ? bupdate_kernel<8> : bupdate_kernel<2>;
+  auto kernel = few_blocks(nupd * row_blocks(prm)) ? bupdate_kernel<kFewSlots> : bupdate_kernel<kManySlots>;
   return launch_pdl(kernel, dim3(nupd, row_blocks(prm)), dim3(kThreads), 0, st, prm, upd, step);
 }
 

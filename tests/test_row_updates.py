@@ -2,7 +2,7 @@
 the rule that picks their form, and the squared-error loss's token rows.
 
 A call with n chains updates 24 n blocks a step: up to 456 (19 chains on 152
-SMs) they are resident together and take their slots eight at a time, beyond
+SMs) they are resident together and take their slots six at a time, beyond
 they take two at a time.  One chain of 2,500 tokens has the most slots, a
 sequence without chunks only copies w0.  The first step's update, which forms
 the row targets, is a form of its own.
