@@ -85,7 +85,7 @@ extern "C" {
                                         the call registered (reported through scal3r_ttt_get_status) */
 
 /* config values */
-#define SCAL3R_FP32         0   /* q,k,v,o float32: plain SIMT path */
+#define SCAL3R_FP32         0   /* q,k,v,o float32: SIMT path        */
 #define SCAL3R_BF16         1   /* q,k,v,o bfloat16: tcgen05 tensor-core path */
 #define SCAL3R_LOSS_DOT     0   /* L = -f(k)^T v  (Eq. 9) */
 #define SCAL3R_LOSS_MSE     1   /* L = 1/2 ||f(k) - v||^2 */
@@ -191,7 +191,7 @@ int scal3r_ttt_forward(scal3r_ttt_handle* handle,
  *   It takes the configuration instead of a handle and no workspace; every
  * other argument means what it means for scal3r_ttt_forward, and the results
  * are those of scal3r_ttt_forward under the schedule this call uses: waves 1,
- * cost ratios 1.85 / 2.25, no tail fill (a bfloat16 handle's default
+ * cost ratios 1.85 / 2.25, no tail fill (a head_dim-64 handle's default
  * schedule sums a chunk's tokens over other pieces, so its results differ
  * in rounding only).  Its scratch (schedule, master weights,
  * partial sums, status word) is one fixed 32 MiB device array inside the
@@ -313,7 +313,8 @@ typedef struct scal3r_ttt_schedule {
                                wave).  The pieces modelled to end first take extra pieces cut off
                                the longest ones, launched behind the first wave; kept for a step
                                only where the library's piece-time model shortens it.  BF16
-                               head_dim-64 path with the dot loss only; ignored elsewhere.
+                               head_dim-64 path with the dot loss only; ignored elsewhere (the
+                               float32 path of that shape always fills, by its own model).
                                Default 3 for a BF16 head_dim-64 handle, else 0; the autotuner
                                tries it on and off.  Results match to rounding: a chunk's
                                token sum is split at other boundaries */

@@ -41,7 +41,7 @@
 //     warps beside 9,600 of MMAs, and two accumulators then bound a tile at half
 //     the sum; eight warps a tile and gate_tile's stores: apply gate 156 -> 144 us,
 //     gradient gate 205 -> 191 us (225 at first), update-VJP gate 485 -> 447 us.
-// Now the tensor pipe is active 70 to 89 %, the SM clock falls to 1.8 GHz under the
+// Now the tensor pipe is active 70 to 89 %, the SM clock falls to 1.7 GHz under the
 // power cap, and rounds of tiles (3.47 run as 4) and the gates' stores beside the
 // operand stream are what is left.
 #include <cudaTypedefs.h>
