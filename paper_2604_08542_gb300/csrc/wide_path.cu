@@ -522,12 +522,14 @@ __device__ __forceinline__ void staged_bkey(const GemmArgs& g, const OutStage& s
 
 // One tile's staged epilogue: accumulator columns acc + cb .. acc + cb + 127 of
 // this warp's 32 lanes, output rows m - lane .. (m: this lane's), columns n0 + cb
-// ..; plane: the K range's partial plane.
+// ..; plane: the K range's partial plane.  A warp without rows fills nothing:
+// where two buffers alternate, "all groups but the newest are read" frees the
+// older one only if every filled buffer is followed by a committed group.
 __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& st, uint32_t acc, int m, int n0, int cb,
                                             int plane) {
   const int row0 = m - st.lane;
+  if (row0 >= g.M) return;
   const bool valid = m < g.M;
-  const bool any = row0 < g.M;   // the warp has rows to store
   if (g.epi == EPI_F32 || g.epi == EPI_F32_ADD || g.epi == EPI_F32_ADDIN) {
     const uint4* xin = nullptr;
     if (g.epi == EPI_F32_ADDIN)
@@ -556,7 +558,7 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
       for (int j = 0; j < 8; ++j)
         st.put(b, j, make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]),
                                    __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3])));
-      if (st.ready() && any) {
+      if (st.ready()) {
         if (g.epi == EPI_F32_ADD) tma_reduce_add_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
         else tma_store_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
         bulk_commit();
@@ -588,7 +590,7 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
           st.put(0, 4 * hh + j, pack8f(x));
         }
       }
-      if (st.ready() && any) {
+      if (st.ready()) {
         tma_store_3d(&g.o[0], st.buf, n0 + c0, row0, 0);
         tma_store_3d(&g.o[1], st.buf + 4096, n0 + c0, row0, 0);
         bulk_commit();
@@ -628,7 +630,7 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
       float* ssq = reinterpret_cast<float*>(g.out[3]) + (size_t)m * g.ld_part + (part * dm + oc + c0) / 64;
       if (in_bounds(ssq, 4)) *ssq = ss;
     }
-    if (st.ready() && any) {
+    if (st.ready()) {
       tma_store_3d(&g.o[part], st.buf + b, oc + c0, row0, 0);
       bulk_commit();
     }
