@@ -312,12 +312,12 @@ typedef struct scal3r_ttt_schedule {
   int32_t tail_fill;        /* 0..3.  Bit 0: forward steps, bit 1: backward steps (each with one
                                wave).  The pieces modelled to end first take extra pieces cut off
                                the longest ones, launched behind the first wave; kept for a step
-                               only where the library's piece-time model shortens it.  BF16
-                               head_dim-64 path with the dot loss only; ignored elsewhere (the
-                               float32 path of that shape always fills, by its own model).
-                               Default 3 for a BF16 head_dim-64 handle, else 0; the autotuner
-                               tries it on and off.  Results match to rounding: a chunk's
-                               token sum is split at other boundaries */
+                               only where the library's piece-time model shortens it.  The
+                               head_dim-64, hidden-128 paths, BF16 (dot loss only) and float32,
+                               each with its own model; ignored elsewhere.  Default 3 for a
+                               handle of that shape, else 0; the autotuner tries it on and off.
+                               Results match to rounding: a chunk's token sum is split at
+                               other boundaries */
 } scal3r_ttt_schedule;
 
 /* Replace / read the handle's schedule.  Setting it drops the cached plan

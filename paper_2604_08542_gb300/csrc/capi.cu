@@ -209,7 +209,6 @@ bool same_layout(const Plan& p, const int64_t* off, int32_t C, const int32_t* pt
 // units of an applied token (forward, 0.2 us on one SM) or an apply-VJP token
 // (backward, 0.5 us); the fixed cost is the weights' load and the sums' store.
 void fp32_fill_model(Schedule& sch) {
-  sch.fill = 3;
   sch.fill_ovh[0] = 40.f;
   sch.fill_ovh[1] = 25.f;
   sch.fill_ovh[2] = 20.f;
@@ -230,8 +229,9 @@ int ensure_plan(scal3r_ttt_handle* hd, const int64_t* off, int32_t C, const int3
     sch.align = 16;
     sch.min_tokens = 16;
   }
+  // the tail fill's model is the BF16 kernels' or, of the same shape, the float32 ones'
   if (hd->cfg.dtype == SCAL3R_FP32 && fp32_tiled_shape(hd->shape.D, hd->shape.F)) fp32_fill_model(sch);
-  else if (hd->cfg.dtype != SCAL3R_BF16 || hd->wide || hd->shape.lin) sch.fill = 0;   // its model is the BF16 kernels'
+  else if (hd->cfg.dtype != SCAL3R_BF16 || hd->wide || hd->shape.lin) sch.fill = 0;
   int rc = build_plan(np, hd->shape, sch, hd->num_sms, off, C, ptr, S, hd->wide ? 1 : hd->cfg.ckpt_every,
                       mse_compose);
   if (rc != SCAL3R_OK) return rc;
@@ -594,6 +594,7 @@ int scal3r_ttt_init(const scal3r_ttt_config* cfg, scal3r_ttt_handle** out) {
     hd->sched.fill = 3;
     hd->sched.key_cost = 2.45f;
   }
+  if (cfg->dtype == SCAL3R_FP32 && !lin && fp32_tiled_shape(cfg->head_dim, cfg->hidden_dim)) hd->sched.fill = 3;
   if (cudaMalloc((void**)&hd->d_status, sizeof(int)) != cudaSuccess ||
       cudaMemset(hd->d_status, 0, sizeof(int)) != cudaSuccess ||
       cudaStreamCreateWithFlags(&hd->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
