@@ -12,7 +12,8 @@
 // uploads it on the call's stream before the call's kernels and uploads an
 // empty table (checking off) after them, so no table outlives its call.
 // TMA loads and stores are not routed through it: the tensor maps bound them
-// in hardware.
+// in hardware.  The wide path's products check the rows of each staged output
+// group before TMA stores it.
 #pragma once
 
 #include <cstdint>

@@ -290,6 +290,36 @@ struct OutStage {
   }
 };
 
+// Row m, column n of output i.
+template <typename T>
+__device__ __forceinline__ T* out_at(const GemmArgs& g, int i, int m, int n) {
+  return reinterpret_cast<T*>(g.out[i]) + (size_t)m * g.ld_out + n;
+}
+
+// Bounds-checking build: whether all of the group's rows (row: this lane's, in
+// global memory; bytes: 128 or 32 a row) lie in a registered range, so that TMA
+// may store them.  If not, the lanes store their rows' 16-byte chunks that do, and
+// the caller commits an empty group.  The whole warp calls it.
+#ifdef SCAL3R_DEBUG_BOUNDS
+__device__ __noinline__ bool group_checked(const OutStage& st, int b, int bytes, void* row, bool valid, bool add) {
+  if (__all_sync(0xffffffffu, !valid || in_bounds(row, bytes))) return true;
+  for (int c = 0; valid && c < bytes / 16; ++c) {
+    const int at = bytes == 128 ? st.lane * 128 + ((c ^ (st.lane & 7)) << 4)
+                                : st.lane * 32 + ((c ^ ((st.lane >> 2) & 1)) << 4);
+    float4* p = reinterpret_cast<float4*>(static_cast<uint8_t*>(row) + 16 * c);
+    float4 x = *reinterpret_cast<const float4*>(st.buf + b + at);
+    if (!in_bounds(p, 16)) continue;
+    if (add) x = make_float4(p->x + x.x, p->y + x.y, p->z + x.z, p->w + x.w);
+    *p = x;
+  }
+  return false;
+}
+#else
+__device__ __forceinline__ constexpr bool group_checked(const OutStage&, int, int, const void*, bool, bool) {
+  return true;
+}
+#endif
+
 __device__ __forceinline__ uint4 pack8f(const float* v) {
   return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
 }
@@ -504,9 +534,14 @@ __device__ __forceinline__ void staged_bkey(const GemmArgs& g, const OutStage& s
 #pragma unroll
       for (int q = 0; q < 6; ++q) st.put32(1024 * q, hh, make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]));
     }
+    uint32_t tma = 0;   // the outputs that TMA stores
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+      tma |= (uint32_t)group_checked(st, 1024 * q, 32, out_at<__nv_bfloat16>(g, q, m, f0 + c), valid, false) << q;
     if (st.ready() && any) {
 #pragma unroll
-      for (int q = 0; q < 6; ++q) tma_store_3d(&g.o[q], st.buf + 1024 * q, f0 + c, row0, 0);
+      for (int q = 0; q < 6; ++q)
+        if (tma >> q & 1) tma_store_3d(&g.o[q], st.buf + 1024 * q, f0 + c, row0, 0);
       bulk_commit();
     }
 #pragma unroll
@@ -558,9 +593,11 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
       for (int j = 0; j < 8; ++j)
         st.put(b, j, make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]),
                                    __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3])));
+      const bool add = g.epi == EPI_F32_ADD;
+      const bool tma = group_checked(st, b, 128, out_at<float>(g, 0, m, n0 + c) + plane * g.split_stride, valid, add);
       if (st.ready()) {
-        if (g.epi == EPI_F32_ADD) tma_reduce_add_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
-        else tma_store_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
+        if (tma && add) tma_reduce_add_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
+        else if (tma) tma_store_3d(&g.o[0], st.buf + b, n0 + c, row0, plane);
         bulk_commit();
       }
     }
@@ -590,9 +627,11 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
           st.put(0, 4 * hh + j, pack8f(x));
         }
       }
+      const bool tma0 = group_checked(st, 0, 128, out_at<__nv_bfloat16>(g, 0, m, n0 + c0), valid, false);
+      const bool tma1 = group_checked(st, 4096, 128, out_at<__nv_bfloat16>(g, 1, m, n0 + c0), valid, false);
       if (st.ready()) {
-        tma_store_3d(&g.o[0], st.buf, n0 + c0, row0, 0);
-        tma_store_3d(&g.o[1], st.buf + 4096, n0 + c0, row0, 0);
+        if (tma0) tma_store_3d(&g.o[0], st.buf, n0 + c0, row0, 0);
+        if (tma1) tma_store_3d(&g.o[1], st.buf + 4096, n0 + c0, row0, 0);
         bulk_commit();
       }
     }
@@ -630,8 +669,9 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
       float* ssq = reinterpret_cast<float*>(g.out[3]) + (size_t)m * g.ld_part + (part * dm + oc + c0) / 64;
       if (in_bounds(ssq, 4)) *ssq = ss;
     }
+    const bool tma = group_checked(st, b, 128, out_at<__nv_bfloat16>(g, part, m, oc + c0), valid, false);
     if (st.ready()) {
-      tma_store_3d(&g.o[part], st.buf + b, oc + c0, row0, 0);
+      if (tma) tma_store_3d(&g.o[part], st.buf + b, oc + c0, row0, 0);
       bulk_commit();
     }
   }
@@ -1594,9 +1634,6 @@ int num_sms() {
 // has no staged form or an output cannot be mapped (its base or row stride is
 // not a multiple of 16 bytes), then the outputs are stored directly.
 bool stage_outputs(GemmArgs& a) {
-#ifdef SCAL3R_DEBUG_BOUNDS
-  return false;   // the checked stores are the direct ones
-#else
   auto fn = encode_fn();
   if (!fn) return false;
   auto map = [&](int i, int64_t cols, int64_t ld, bool f32, int box_cols, int64_t planes,
@@ -1630,7 +1667,6 @@ bool stage_outputs(GemmArgs& a) {
       return true;
     default: return false;
   }
-#endif
 }
 
 // The weight maps of a gate product for gate_tile: the hidden units of every 32
