@@ -1671,22 +1671,26 @@ bool stage_outputs(GemmArgs& a) {
 
 // The weight maps of a gate product for gate_tile: the hidden units of every 32
 // reordered (a 5-D view of the matrix whose box walks them as p, t, j of
-// f = 8 t + 2 j + p).  False if this is no gate product of that form.
+// f = 8 t + 2 j + p).  False, and b[] as it was, if this is no gate product of
+// that form or a map cannot be encoded.
 bool gate_maps(GemmArgs& a) {
   const bool gate = a.epi == EPI_KEY || a.epi == EPI_BAPPLY || a.epi == EPI_APPLY;
   auto fn = encode_fn();
   if (!gate || !fn || !a.bw[0] || a.nbn != 2) return false;
   const cuuint64_t row = (cuuint64_t)a.K * 2;
-  for (int i = 0; i < a.nbn; ++i) {
+  CUtensorMap m[2];
+  for (int i = 0; i < 2; ++i) {
     cuuint64_t dims[5] = {(cuuint64_t)a.K, 2, 4, 4, (cuuint64_t)(a.b_rows / 32)};
     cuuint64_t strides[4] = {row, 8 * row, 2 * row, 32 * row};
     cuuint32_t box[5] = {64, 2, 4, 4, BN / 2 / 32};
     cuuint32_t es[5] = {1, 1, 1, 1, 1};
-    if (fn(&a.b[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.bw[i]), dims, strides, box, es,
+    if (fn(&m[i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(a.bw[i]), dims, strides, box, es,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return false;
   }
+  a.b[0] = m[0];
+  a.b[1] = m[1];
   a.gated = 1;
   return true;
 }
