@@ -38,9 +38,14 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# the current stream without building a Stream object; torch's own, so possibly not in every version
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(dev) -> int:
-    # torch.cuda.current_stream(dev).cuda_stream without building a Stream object
-    return torch._C._cuda_getCurrentRawStream(dev.index)
+    if dev.type != "cuda":
+        raise ValueError(f"Expected a cuda device, but got: {dev}")
+    return torch.cuda.current_stream(dev).cuda_stream if _raw_stream is None else _raw_stream(dev.index)
 
 
 class _Layout:
