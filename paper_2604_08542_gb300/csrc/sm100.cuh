@@ -174,7 +174,8 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void*
                : "memory");
 }
 
-// The tile added to global memory (the map's element type).
+// The tile added to global memory (the map's element type; float32 adds keep
+// subnormals on GB300, as a load, an add and a store do: test_gemm_accumulate.py).
 __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* map, const void* ssrc, int32_t c0, int32_t c1,
                                                   int32_t c2) {
   asm volatile("cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
