@@ -206,8 +206,18 @@ bool same_layout(const Plan& p, const int64_t* off, int32_t C, const int32_t* pt
 }
 
 // The tail fill's piece-time model for the register-tiled float32 kernels, in
-// units of an applied token (forward, 0.2 us on one SM) or an apply-VJP token
-// (backward, 0.5 us); the fixed cost is the weights' load and the sums' store.
+// units of an applied token (forward, 0.182 us on one SM) or an apply-VJP token
+// (backward, 0.479 us); the fixed cost is the weights' load and the sums' store.
+// One piece of n tokens alone on the GPU, 64 to 4096 tokens, fits within 0.7 % (us):
+//   gradient   7.2 + 0.326 n   (squared error  7.3 + 0.442 n)
+//   apply      3.3 + 0.182 n
+//   update VJP 7.1 + 0.924 n   (squared error  7.2 + 1.591 n)
+//   apply VJP  5.3 + 0.479 n
+// that is 40 + 1.79 n and 18 + n forward, 15 + 1.93 n and 11 + n backward; the
+// constants below were set before that fit, and price the fixed costs a little high.
+// They are the dot loss's; the fill pays with the squared error all the same.  Without
+// -> with the fill, 16 heads, two sequences of two chunks of 2,082 tokens: forward
+// 707 -> 558 us, backward 1824 -> 1425 (squared error 893 -> 697, 2336 -> 2243).
 void fp32_fill_model(Schedule& sch) {
   sch.fill_ovh[0] = 40.f;
   sch.fill_ovh[1] = 25.f;

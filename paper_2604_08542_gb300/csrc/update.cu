@@ -82,8 +82,10 @@ __device__ __forceinline__ float normsq4(float4 a) {                        // o
 
 // The two update kernels exist twice.  A grid whose blocks are all resident at
 // three a SM (16 chains of the (64, 128) layer: 384 blocks) waits for memory
-// round trips only, and takes its slots six at a time in 70 to 78 registers
-// (eight at a time spill, 0.4 % of a 256-frame training step).  A larger one
+// round trips only, and takes its slots six at a time in 70 to 78 registers.
+// (Eight at a time spill: 16 chains' update 8.3 -> 9.2 us, its adjoint's 8.4 -> 10.0,
+// the 256-frame training step 3613 -> 3626 us, four alternating runs of each within
+// 1 us.  Four at a time: 3620 us.)  A larger one
 // needs warps in flight: two slots at a time, so that eight blocks (the
 // backward's: six) fit a SM.  The update of 352 chains took 38 us with eight at a
 // time and takes 24.5 (at 100 MB, 4.2 TB/s), of 32 chains 6.8 and 6.0.

@@ -41,9 +41,11 @@
 //     warps beside 9,600 of MMAs, and two accumulators then bound a tile at half
 //     the sum; eight warps a tile and gate_tile's stores: apply gate 156 -> 144 us,
 //     gradient gate 205 -> 191 us (225 at first), update-VJP gate 485 -> 447 us.
-// Now the tensor pipe is active 70 to 89 %, the SM clock falls to 1.7 GHz under the
-// power cap, and rounds of tiles (3.47 run as 4) and the gates' stores beside the
-// operand stream are what is left.
+// Now the tensor pipe is active 83 to 92 % in the launches with K of 4096 and more, which
+// run at what cuBLAS sustains under the power cap (1.72 of 1.74 PFLOP/s; SM clock 1.54 to
+// 1.70 GHz in a loop), 70 to 72 % in the products with K = 1024, 69 % in the gradient and
+// apply-VJP gates (83 % in the apply gate) and 59 % in the update-VJP gate: the stores of
+// outputs beside the operand stream and rounds of tiles (3.47 run as 4) are what is left.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -225,13 +227,6 @@ __device__ __forceinline__ uint4 ldg16(const uint4* p) {
     if ((p) && !in_bounds((p), (uint32_t)(bytes))) return;   \
   } while (0)
 
-// Persistent: CTA b takes output tiles b, b + gridDim.x, ... (consecutive
-// CTAs share an A row-block).  The TMA warp runs the stage ring across tiles;
-// the MMA warp alternates between two 256-column accumulators; epilogue group
-// g (four warps, all 128 TMEM lanes) drains the tiles of accumulator g, so a
-// tile's epilogue overlaps the next tile's MMAs.
-// XSET: the update-VJP gate and the squared-error loss's epilogues, in their own
-// instantiation so that the common ones keep their register allocation.
 // The three learning rates of output row m (W1, W3, W2).
 __device__ __forceinline__ void row_rates(const GemmArgs& g, int m, float& e1, float& e3, float& e2) {
   const float* ep = g.eta + (size_t)m * g.eta_stride;
@@ -679,6 +674,19 @@ __device__ __forceinline__ void staged_tile(const GemmArgs& g, const OutStage& s
 
 constexpr int group_max(bool xset, bool pair) { return pair && !xset ? kMaxGroup : 1; }
 
+// Persistent: CTA (or pair) b takes work units b, b + their number, ... of the
+// launch's products (consecutive ones share an A row block).  Two TMA warps run the
+// stage ring across units, A's and B's; one warp issues the MMAs into two
+// 256-column accumulators in turn; a unit's epilogue runs under the next one's MMAs.
+// Arrivals a phase:
+//   full       1: the A producer (the even CTA's) expects all of the stage's bytes
+//   empty      1: the commit of the stage's MMAs, in both CTAs of a pair
+//   acc_full   1: the commit of a unit's last MMA, in both CTAs of a pair
+//   acc_empty  the warps that drain the accumulator, of both CTAs of a pair, on the
+//              even CTA's barrier: all eight (each group half of the columns), or,
+//              XSET, the four of the group whose accumulator it is.
+// XSET: the update-VJP gate and the squared-error loss's epilogues, in their own
+// instantiation so that the common ones keep their register allocation.
 template <bool XSET, bool PAIR>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     wide_gemm_kernel(const __grid_constant__ GemmGroup<group_max(XSET, PAIR)> grp) {
@@ -1696,7 +1704,18 @@ bool gate_maps(GemmArgs& a) {
 }
 
 // CTA pairs or single CTAs: the fewer rounds of tiles, a pair's round (256 x
-// 256 outputs on two SMs) counted 0.9 of a single's (128 x 256 on each).
+// 256 outputs on two SMs) counted 0.9 of a single's (128 x 256 on each).  Both forms
+// on GB300, M x N x K, rounds single / pairs, us single -> pairs, bf16 | float32 out:
+//   2432 x 2048 x 1024     1 / 2    12.8 -> 18.8 | 16.3 -> 20.8   single is taken
+//   7200 x 2048 x 4096     3 / 4    76.0 -> 82.6 | 84.7 -> 86.8   single
+//   16656 x 4096 x 1024   14 / 14   97.4 -> 94.5 | 153.4 -> 112.9 pairs
+//   16656 x 1024 x 4096    4 / 4    99.5 -> 89.2 | 110.7 -> 93.3  pairs
+//   4096 x 1024 x 16656    1 / 1    106.9 -> 87.6 | 110.5 -> 89.0 pairs
+//   4164 x 1024 x 4096     1 / 1    25.1 -> 27.0 | 28.8 -> 27.1   pairs
+//   600 x 1024 x 1024      1 / 1    12.6 -> 13.1 | 14.6 -> 14.7   pairs
+//   2433 x 2048 x 1024     2 / 2    16.7 -> 18.8 | 19.1 -> 20.7   pairs
+// So 0.9 is the gain of several rounds (0.81 to 0.97); a bf16 output of one or two
+// short rounds runs up to 13 % longer on pairs, as the last three show.
 bool use_pairs(int M, int64_t units, int64_t pairs, int64_t sms) {
   if (M <= BM || sms < 2) return false;   // one row block: the pair's other half would be empty
   const int64_t r1 = (units + sms - 1) / sms, r2 = (pairs + sms / 2 - 1) / (sms / 2);
