@@ -1708,18 +1708,34 @@ bool gate_maps(GemmArgs& a) {
 // on GB300, M x N x K, rounds single / pairs, us single -> pairs, bf16 | float32 out:
 //   2432 x 2048 x 1024     1 / 2    12.8 -> 18.8 | 16.3 -> 20.8   single is taken
 //   7200 x 2048 x 4096     3 / 4    76.0 -> 82.6 | 84.7 -> 86.8   single
-//   16656 x 4096 x 1024   14 / 14   97.4 -> 94.5 | 153.4 -> 112.9 pairs
-//   16656 x 1024 x 4096    4 / 4    99.5 -> 89.2 | 110.7 -> 93.3  pairs
 //   4096 x 1024 x 16656    1 / 1    106.9 -> 87.6 | 110.5 -> 89.0 pairs
-//   4164 x 1024 x 4096     1 / 1    25.1 -> 27.0 | 28.8 -> 27.1   pairs
-//   600 x 1024 x 1024      1 / 1    12.6 -> 13.1 | 14.6 -> 14.7   pairs
-//   2433 x 2048 x 1024     2 / 2    16.7 -> 18.8 | 19.1 -> 20.7   pairs
-// So 0.9 is the gain of several rounds (0.81 to 0.97); a bf16 output of one or two
-// short rounds runs up to 13 % longer on pairs, as the last three show.
+//   16656 x 1024 x 4096    4 / 4    99.5 -> 89.2 | 110.7 -> 93.3  pairs
+//   16656 x 4096 x 1024   14 / 14   97.4 -> 94.5 | 153.4 -> 112.9 pairs
+// A float32 output gains from the staged stores at any length; a bf16 one does not
+// (see short_bf16).
 bool use_pairs(int M, int64_t units, int64_t pairs, int64_t sms) {
   if (M <= BM || sms < 2) return false;   // one row block: the pair's other half would be empty
   const int64_t r1 = (units + sms - 1) / sms, r2 = (pairs + sms / 2 - 1) / (sms / 2);
   return 10 * r1 > 9 * r2;
+}
+
+// A product with bf16 outputs that is too short for pairs.  They cost a launch 0.6 to
+// 1.5 us more (the cluster's barriers, the staging), and pay through the operand bytes
+// they save: where a tile has 12 K blocks and more and the launch 64 rounds of them, or
+// where one column of tiles streams an A beyond half of the L2.  Graph replays on GB300,
+// us single -> pairs:
+//   130 x 256 x 64       4.7 -> 6.0     5000 x 1024 x 64      6.7 -> 8.7   single is taken
+//   4164 x 1024 x 1024  10.3 -> 11.2    2082 x 1024 x 2048   13.5 -> 14.9  single
+//   16656 x 4096 x 512  56.4 -> 59.4    8328 x 1024 x 2048   24.9 -> 25.0  single, pairs (64)
+//   4164 x 4096 x 1024  27.4 -> 26.8    16656 x 2048 x 768   40.3 -> 38.3  pairs (64, 84)
+//   16656 x 1024 x 2048 52.9 -> 49.2    50000 x 256 x 1024   32.0 -> 28.4  pairs (128; A 102 MB)
+// Over 396 products of 130 to 50,000 rows this takes the slower form by 5 % or more in
+// five, by 8 % at most (pairs for bf16 at every length: in 198, by 38 %).
+bool short_bf16(const GemmArgs& a, int64_t pairs, int64_t sms) {
+  if (a.epi != EPI_BF16 && a.epi != EPI_GCM_QKV && a.epi != EPI_GCM_GATE) return false;
+  const int64_t nk = (a.K + BK - 1) / BK, rounds = (pairs + sms / 2 - 1) / (sms / 2);
+  const bool streams = a.N == BN && nk >= 16 && (int64_t)a.M * a.K * 2 >= (int64_t)64 << 20;
+  return !streams && (nk < 12 || rounds * nk < 64);
 }
 
 template <int NG>
@@ -1764,7 +1780,7 @@ cudaError_t gemm(GemmArgs& a, cudaStream_t st) {
   const cudaError_t e = complete(a, units, pairs);
   if (e != cudaSuccess) return e;
   const bool xset = (a.epi >= EPI_MSE_E && a.epi <= EPI_APPLY2) || a.epi == EPI_BKEY;
-  if (use_pairs(a.M, units, pairs, num_sms()) && (gate_maps(a) || (a.staged = stage_outputs(a)) || xset)) {
+  if (use_pairs(a.M, units, pairs, num_sms()) && !short_bf16(a, pairs, num_sms()) && (gate_maps(a) || (a.staged = stage_outputs(a)) || xset)) {
     if (xset) return launch_pairs(wide_gemm_kernel<true, true>, GemmGroup<1>{{a}, {0, (int)pairs}, 1}, st);
     return launch_pairs(wide_gemm_kernel<false, true>, GemmGroup<kMaxGroup>{{a}, {0, (int)pairs}, 1}, st);
   }

@@ -1,7 +1,10 @@
 """The bounds-checking build launches the kernels of the ordinary one (GPU): the
 same forward and backward of a wide layer, captured into a graph in one process
 per build, has the same product launches (grid, block and shared memory: CTA pairs
-and single CTAs differ in each), pairs among them."""
+and single CTAs differ in each), pairs among them.
+
+A violation planted in a staged output (o registered 32 bytes short, see
+test_bounds_build.py) is reported, and only the 16 outputs outside are left out."""
 import ctypes
 import json
 import os
@@ -61,9 +64,31 @@ def _child():
             layer.backward(*args, g["d_o"], ck, wn, workspace=ws, out=grads)
 
         launches = _captured_launches(s.cuda_stream, step)
+    planted = _planted() if ttt.LIB_PATH.endswith("_bounds.so") else None
     # 11 warps: the product kernel
     print(json.dumps({"library": ttt.LIB_PATH, "status": layer.status(),
-                      "products": [d for d in launches if d[3] == 352]}))
+                      "products": [d for d in launches if d[3] == 352], "planted": planted}))
+
+
+def _planted():
+    """o = h W2^T over hidden 4096 runs as a pair with staged outputs."""
+    import torch
+    import paper_2604_08542_gb300 as ttt
+    import ttt_synth as syn
+    from _util import upload
+    H, D, F = 1, 256, 4096
+    lay = syn.layout_from_lengths([[200]])
+    g = upload(syn.make_inputs(lay.num_tokens, H, D, F, seed=32, dtype="bf16"), torch.bfloat16)
+    layer = ttt.TTT(H, D, F, dtype=torch.bfloat16)
+    args = (g["q"], g["k"], g["v"], g["lr"], g["w0"], lay.chunk_offsets, lay.seq_chunk_ptr)
+    ref = layer.forward(*args)[0].reshape(-1)
+    o = torch.full_like(g["q"], 7.0)
+    ttt.scal3r_ttt_debug_bounds(layer.handle, 5, 32)   # o
+    layer.forward(*args, o=o)
+    torch.cuda.synchronize()
+    flat = o.reshape(-1)
+    return {"status": layer.status(), "tail_untouched": bool((flat[-16:] == 7.0).all()),
+            "rest_written": bool(torch.equal(flat[:-16], ref[:-16]))}
 
 
 @pytest.mark.gpu
@@ -79,5 +104,7 @@ def test_bounds_build_runs_the_same_product_kernels():
         out = json.loads(r.stdout.strip().splitlines()[-1])
         assert out["library"] == lib and out["status"] == 0
         got.append(out["products"])
+        planted = out["planted"]
     assert 230400 in {d[6] for d in got[0]}   # pairs: five 32 KB stages, 64 KB of staged outputs, 1 KB
     assert got[1] == got[0]
+    assert planted == {"status": 9, "tail_untouched": True, "rest_written": True}   # SCAL3R_ERR_BOUNDS
